@@ -74,8 +74,8 @@
  * call fails with EF_ERR_TIMEOUT (reported by ef_check_status); it never
  * hangs and never returns a wrong result. From 4096 tiles on, the streaming
  * kernel's CTAs claim groups of tiles in the order they start, and the
- * one-tile-per-CTA path (misaligned g or e, ef_hard_threshold_noalloc) takes
- * its tiles the same way: neither needs co-residency.
+ * one-tile-per-CTA kernel (ef_hard_threshold_noalloc) takes its tiles the same
+ * way: neither needs co-residency.
  */
 #ifndef EFSPARSE_H
 #define EFSPARSE_H
@@ -113,8 +113,8 @@ typedef enum {
  *
  *   g          [in]  fp32[d], the stochastic gradient g_{i,t}. 4-byte aligned.
  *   e          [in/out] fp32[d], the error memory e_{i,t}; overwritten with
- *                    e_{i,t+1} = a - C(a). 4-byte aligned; 16-byte alignment of
- *                    both g and e selects the vectorised path.
+ *                    e_{i,t+1} = a - C(a). 4-byte aligned (any such g and e
+ *                    stream at the same speed but for a few per cent).
  *   gamma      step size; must be finite.
  *   lambda     threshold; must be >= 0 and not NaN (+inf sends only +-inf).
  *   d          number of coordinates, 0 <= d <= 2^32 - 1.
@@ -132,8 +132,7 @@ ef_status ef_hard_threshold(const float* g, float* e, float gamma, float lambda,
 
 /*
  * ef_hard_threshold_bf16 — as ef_hard_threshold, with the gradient stored as
- * bfloat16 bit patterns (uint16_t[d], 2-byte aligned; 8-byte alignment of g
- * and 16-byte alignment of e select the vectorised path). Each g[j] is widened
+ * bfloat16 bit patterns (uint16_t[d], 2-byte aligned). Each g[j] is widened
  * exactly to fp32 (its 16 bits become the high half of the fp32 word) before
  * the same fused multiply-add; all other semantics are identical.
  */
@@ -229,8 +228,7 @@ ef_status ef_topk_layerwise_bf16(const uint16_t* g, float* e, float gamma, uint3
  * (nonnegative terms), plus the squares below the fp32 range
  * (|e'_j| < 2^-75), which contribute 0; a sum beyond the fp32 range
  * (|e'_j| >= 2^64 suffices) makes it +inf. It is bit-for-bit reproducible for a given device and input.
- * The streaming kernels add it as they go; steps whose g or e are not
- * 16-byte aligned compute it with one more pass over e'. After a step that
+ * The streaming kernels add it as they go. After a step that
  * failed on the device (a latched timeout) it holds a NaN.
  */
 ef_status ef_hard_threshold_ex(const void* g, ef_grad_type g_type, float* e, float gamma,
@@ -459,7 +457,7 @@ void ef_test_set_lookback_fault(int64_t withheld_tile, uint32_t spin_limit_us);
 /*
  * ef_test_set_stream_kernel — test hook choosing the streaming kernel of the
  * hard-threshold step and of the Top-k and layer-wise Top-k candidate passes
- * (16-byte aligned g and e): 0 (the default) by size (claimed groups of tiles
+ * (g and e at any alignment): 0 (the default) by size (claimed groups of tiles
  * with look-back from 4096 tiles, 16,777,216 coordinates, on; static chunks
  * below; for the hard-threshold step, a shallower ring with larger pair
  * buffers once an earlier call on the same stream sent at least 1/12 of its

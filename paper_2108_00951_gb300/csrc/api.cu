@@ -181,8 +181,8 @@ ef_status hard_threshold_entry(const void* g, bool bf16, float* e, float gamma, 
   ef_status st = device_info(dev, &info);
   if (st != EF_OK) return st;
   Workspace* ws = nullptr;
-  st = acquire_workspace(stream, tiles_for(d), 0, 0,
-                         static_cast<size_t>(tiles_for(d)) * kTileElems, &ws);
+  st = acquire_workspace(stream, stream_tiles_for(d), 0, 0,
+                         static_cast<size_t>(stream_tiles_for(d)) * kTileElems, &ws);
   if (st != EF_OK) return st;
   return finish_launch(launch_hard_threshold(g, bf16, e, gamma, lambda, static_cast<uint32_t>(d),
                                              idx_out, val_out, count_out, err_out, tiles_out, *ws,
@@ -221,8 +221,8 @@ ef_status topk_entry(const void* g, bool bf16, float* e, float gamma, uint64_t k
   ef_status st = device_info(dev, &info);
   if (st != EF_OK) return st;
   Workspace* ws = nullptr;
-  st = acquire_workspace(stream, tiles_for(d), topk_candidate_capacity(d), 0,
-                         static_cast<size_t>(tiles_for(d)) * kTileElems, &ws);
+  st = acquire_workspace(stream, stream_tiles_for(d), topk_candidate_capacity(d), 0,
+                         static_cast<size_t>(stream_tiles_for(d)) * kTileElems, &ws);
   if (st != EF_OK) return st;
   if (err_out && (overlaps(err_out, 8, e, nb) || overlaps(err_out, 8, g, d * gsz) ||
                   overlaps(err_out, 8, idx_out, kb) || overlaps(err_out, 8, val_out, kb) ||
@@ -274,8 +274,8 @@ ef_status topk_layerwise_entry(const void* g, bool bf16, float* e, float gamma, 
   ef_status st = device_info(dev, &info);
   if (st != EF_OK) return st;
   Workspace* ws = nullptr;
-  st = acquire_workspace(stream, tiles_for(d), topk_candidate_capacity(d), 0,
-                         static_cast<size_t>(tiles_for(d)) * kTileElems, &ws);
+  st = acquire_workspace(stream, stream_tiles_for(d), topk_candidate_capacity(d), 0,
+                         static_cast<size_t>(stream_tiles_for(d)) * kTileElems, &ws);
   if (st != EF_OK) return st;
   if (err_out && (overlaps(err_out, 8, e, nb) || overlaps(err_out, 8, g, d * gsz) ||
                   overlaps(err_out, 8, idx_out, kb) || overlaps(err_out, 8, val_out, kb) ||

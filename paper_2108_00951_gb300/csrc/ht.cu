@@ -8,8 +8,9 @@
 // and writes the selected (j, a_j) pairs in ascending j through the ordered
 // compaction. HBM traffic per coordinate is the algorithmic minimum: read g
 // (4 B, or 2 B for bf16) and e (4 B), write e (4 B); plus 8 B per sent pair.
+#include <algorithm>
+
 #include "compact.cuh"
-#include "gradient.cuh"
 #include "internal.h"
 #include "stream_lookback.cuh"
 
@@ -20,9 +21,11 @@ __device__ __forceinline__ uint32_t in_support(float a, float lambda) {
   return (fabsf(a) >= lambda && a != 0.0f) ? 1u : 0u;
 }
 
-template <typename GT, bool kVec>
+// One tile per CTA with the decoupled look-back of compact.cuh: the
+// allocation-free entry's kernel (its scratch is one status word per tile).
+template <bool kVec>
 __global__ void __launch_bounds__(kThreads)
-    ht_kernel(const GT* __restrict__ g, float* __restrict__ e, float gamma, float lambda,
+    ht_kernel(const float* __restrict__ g, float* __restrict__ e, float gamma, float lambda,
               uint32_t d, uint32_t* __restrict__ idx_out, float* __restrict__ val_out,
               uint32_t* __restrict__ count_out, ScanCtx ctx) {
   // The tile comes from the dispenser, in the order CTAs start, so every
@@ -51,7 +54,7 @@ __global__ void __launch_bounds__(kThreads)
   const bool full_tile = static_cast<uint64_t>(tile + 1) * kTileElems <= d;
 
   if (kVec && full_tile) {
-    GradVec<GT> gv[kUnits];
+    GradVec<float> gv[kUnits];
     float4 ev[kUnits];
 #pragma unroll
     for (int v = 0; v < kUnits; ++v) {  // all loads in flight before any use
@@ -103,55 +106,28 @@ __global__ void __launch_bounds__(kThreads)
 // The hard-threshold step as a streaming-compaction op: a stage holds a
 // tile of g followed by the same tile of e; the residual is written to e from
 // registers with streaming stores.
-template <typename GT>
-struct HtOp {
-  const GT* g;
-  float* e;
+template <typename GT, bool kAny>
+struct HtOp : StreamIn<GT, kAny> {
   float gamma, lambda;
-  uint32_t d;
-  static constexpr uint32_t kGBytes = kTileElems * sizeof(GT);
-  static constexpr uint32_t kStageBytes = kGBytes + kTileElems * sizeof(float);
   static constexpr uint32_t kWarpStagePairs = 768;  // on-chip staged pairs per compute warp
   static constexpr bool kKeepPairs = false;  // the message: read by the exchange, much later
-  __device__ void prologue() const {}
-  __device__ uint64_t initial_aux() const { return 0; }
-
   // the chunk's first tiles of g and e toward L2 before the wait for the
   // previous kernel (its tail leaves DRAM mostly idle)
   static constexpr uint32_t kPrefetchTiles = 8;
-  __device__ __forceinline__ void prefetch(uint32_t t) const {
-    prefetch_l2_1d(g + static_cast<size_t>(t) * kTileElems, kGBytes);
-    prefetch_l2_1d(e + static_cast<size_t>(t) * kTileElems, kTileElems * sizeof(float));
-  }
-  __device__ __forceinline__ void fill(unsigned char* stage, uint32_t t, uint64_t* bar,
-                                       uint64_t policy) const {
-    tma_load_1d(stage, g + static_cast<size_t>(t) * kTileElems, kGBytes, bar, policy);
-    tma_load_1d(stage + kGBytes, e + static_cast<size_t>(t) * kTileElems,
-                kTileElems * sizeof(float), bar, policy);
-  }
+  __device__ void prologue() const {}
+  __device__ uint64_t initial_aux() const { return 0; }
 
   __device__ __forceinline__ void tile_smem(const unsigned char* stage, uint32_t t, int warp,
                                             int lane, float (&a)[kSUnits][4],
                                             uint32_t (&sel)[kSUnits], uint64_t) const {
-    const GT* gs = reinterpret_cast<const GT*>(stage);
-    const float* es = reinterpret_cast<const float*>(stage + kGBytes);
     const int local = warp * kSWarpElems + lane * 4;
-    float* eg = e + stream_element_index(t, warp, 0, lane, 0);
+    float* eg = this->e + stream_element_index(t, warp, 0, lane, 0);
     // with lambda > 0, |a| >= lambda already excludes a == 0 (and NaN): one
     // comparison a coordinate; lambda == 0 keeps the a != 0 test
     const bool pos = lambda > 0.0f;
 #pragma unroll
     for (int v = 0; v < kSUnits; ++v) {
-      GradVec<GT> gv;
-      if constexpr (sizeof(GT) == 4)
-        gv.v = *reinterpret_cast<const float4*>(gs + local + v * 128);
-      else
-        gv.v = *reinterpret_cast<const uint2*>(gs + local + v * 128);
-      const float4 ev = *reinterpret_cast<const float4*>(es + local + v * 128);
-      a[v][0] = __fmaf_rn(gamma, gv[0], ev.x);
-      a[v][1] = __fmaf_rn(gamma, gv[1], ev.y);
-      a[v][2] = __fmaf_rn(gamma, gv[2], ev.z);
-      a[v][3] = __fmaf_rn(gamma, gv[3], ev.w);
+      this->accumulate(stage, local + v * 128, gamma, a[v]);
       bool s[4];
 #pragma unroll
       for (int j = 0; j < 4; ++j)
@@ -173,12 +149,12 @@ struct HtOp {
       for (int j = 0; j < 4; ++j) {
         const uint64_t i = first + v * 128 + j;
         a[v][j] = 0.0f;
-        if (i < d) {
-          const float x = __fmaf_rn(gamma, grad_scalar(g, i), e[i]);
+        if (this->valid(i)) {
+          const float x = this->accumulate_at(i, gamma);
           const uint32_t sj = in_support(x, lambda);
           a[v][j] = x;
           sel[v] |= sj << j;
-          e[i] = sj ? 0.0f : x;
+          this->e[i] = sj ? 0.0f : x;
         }
       }
     }
@@ -190,10 +166,10 @@ struct HtOp {
 template <typename GT>
 constexpr int kHtStages = sizeof(GT) == 2 ? 5 : 4;
 
-template <typename GT, int kStages = kHtStages<GT>>
-using HtGroupKernel = LbLayout<HtOp<GT>, kStages>;
-template <typename GT>
-using HtChunkKernel = StreamLayout<HtOp<GT>, kHtStages<GT>>;
+template <typename GT, bool kAny, int kStages = kHtStages<GT>>
+using HtGroupKernel = LbLayout<HtOp<GT, kAny>, kStages>;
+template <typename GT, bool kAny>
+using HtChunkKernel = StreamLayout<HtOp<GT, kAny>, kHtStages<GT>>;
 
 // Streaming hard-threshold over dynamically claimed groups of tiles: one CTA
 // per SM. A group waits only for groups claimed before it, held by running
@@ -201,13 +177,13 @@ using HtChunkKernel = StreamLayout<HtOp<GT>, kHtStages<GT>>;
 // the previous kernel on the stream finishes (the kernel waits for it before
 // its first read). kStages: the ring depth (one stage fewer for dense calls,
 // whose pair buffers then take the freed shared memory).
-template <typename GT, int kStages>
-cudaError_t launch_groups(const GT* g, float* e, float gamma, float lambda, uint32_t d,
+template <int kStages, typename GT, bool kAny>
+cudaError_t launch_groups(const StreamIn<GT, kAny>& in, float gamma, float lambda, uint32_t d,
                           uint32_t* idx_out, float* val_out, uint32_t* count_out, double* err_out,
                           uint32_t* tiles_out, Workspace& ws, const DeviceInfo& dev,
                           const ScanCtx& ctx, int per_sm) {
-  const uint32_t tiles = tiles_for(d);
-  HtOp<GT> op{g, e, gamma, lambda, d};
+  HtOp<GT, kAny> op{in, gamma, lambda};
+  const uint32_t tiles = ctx.num_tiles;
   const uint32_t groups = (tiles + kLbGroupTiles - 1) / kLbGroupTiles;
   const uint32_t slots = static_cast<uint32_t>(per_sm * dev.sm_count);
   const uint32_t grid = groups < slots ? groups : slots;
@@ -216,10 +192,10 @@ cudaError_t launch_groups(const GT* g, float* e, float gamma, float lambda, uint
   // the groups' shares of ||e'||^2 use the per-tile count area (16 words a tile)
   LbArgs la{tiles_out, err_out, reinterpret_cast<FF*>(ws.counts()), ws.stage_idx(),
             ws.stage_val(), ws.density_dev};
-  void* params[] = {&op, &d, &idx_out, &val_out, &count_out, &cap, &c, &la};
+  void* params[] = {&op, &idx_out, &val_out, &count_out, &cap, &c, &la};
   const cudaError_t err = launch_pdl(
-      reinterpret_cast<const void*>(&lookback_stream_kernel<HtOp<GT>, kStages>), grid,
-      kLbThreads, HtGroupKernel<GT, kStages>::kSmem, ws.stream, params, false);
+      reinterpret_cast<const void*>(&lookback_stream_kernel<HtOp<GT, kAny>, kStages>), grid,
+      kLbThreads, HtGroupKernel<GT, kAny, kStages>::kSmem, ws.stream, params, false);
   count_launch();
   ws.ht_part_ready = false;  // the chunk kernel's boundaries are not written by this kernel
   return err;
@@ -234,13 +210,13 @@ cudaError_t launch_groups(const GT* g, float* e, float gamma, float lambda, uint
 // call's chunk boundaries from its chunk totals (dense regions get fewer
 // tiles); any boundaries partition the tiles, so the result never depends on
 // them.
-template <typename GT>
-cudaError_t launch_chunks(const GT* g, float* e, float gamma, float lambda, uint32_t d,
+template <typename GT, bool kAny>
+cudaError_t launch_chunks(const StreamIn<GT, kAny>& in, float gamma, float lambda, uint32_t d,
                           uint32_t* idx_out, float* val_out, uint32_t* count_out, double* err_out,
                           uint32_t* tiles_out, Workspace& ws, const DeviceInfo& dev,
                           const ScanCtx& ctx, int per_sm) {
-  const uint32_t tiles = tiles_for(d);
-  HtOp<GT> op{g, e, gamma, lambda, d};
+  HtOp<GT, kAny> op{in, gamma, lambda};
+  const uint32_t tiles = ctx.num_tiles;
   uint32_t slots = static_cast<uint32_t>(per_sm * dev.sm_count);
   if (slots > kMaxChunks) slots = kMaxChunks;
   const uint32_t grid = tiles < slots ? tiles : slots;
@@ -257,10 +233,10 @@ cudaError_t launch_chunks(const GT* g, float* e, float gamma, float lambda, uint
   sa.prev_part = same && ws.ht_prev_balanced ? ws.ht_part(seq + 2) : nullptr;  // seq - 1
   sa.prev_epoch = ws.ht_last_epoch;
   sa.part_out = ws.ht_part(seq + 1);
-  void* params[] = {&op, &d, &idx_out, &val_out, &count_out, &cap, &c, &sa};
+  void* params[] = {&op, &idx_out, &val_out, &count_out, &cap, &c, &sa};
   const cudaError_t err = launch_pdl(
-      reinterpret_cast<const void*>(&stream_compact_kernel<HtOp<GT>, kHtStages<GT>>), grid,
-      kStreamThreads, HtChunkKernel<GT>::kSmem, ws.stream, params, false);
+      reinterpret_cast<const void*>(&stream_compact_kernel<HtOp<GT, kAny>, kHtStages<GT>>), grid,
+      kStreamThreads, HtChunkKernel<GT, kAny>::kSmem, ws.stream, params, false);
   count_launch();
   ws.ht_prev_balanced = sa.part_in != nullptr;
   ws.ht_part_ready = err == cudaSuccess;
@@ -271,47 +247,37 @@ cudaError_t launch_chunks(const GT* g, float* e, float gamma, float lambda, uint
   return err;
 }
 
-template <typename GT>
+template <bool kAny, typename GT>
 cudaError_t launch_typed(const GT* g, float* e, float gamma, float lambda, uint32_t d,
                          uint32_t* idx_out, float* val_out, uint32_t* count_out, double* err_out,
                          uint32_t* tiles_out, Workspace& ws, const DeviceInfo& dev) {
-  const uint32_t tiles = tiles_for(d);
+  const StreamIn<GT, kAny> in = stream_in<GT, kAny>(g, e, d);
+  const uint32_t tiles = tiles_for(in.end);
   const ScanCtx ctx = next_scan_ctx(ws, tiles);
-  const uintptr_t ga = reinterpret_cast<uintptr_t>(g), ea = reinterpret_cast<uintptr_t>(e);
-  if (ga % 16 == 0 && ea % 16 == 0) {
-    const int per_group = sizeof(GT) == 4 ? dev.ht_group_per_sm_f32 : dev.ht_group_per_sm_bf16;
-    const int per_dense = sizeof(GT) == 4 ? dev.ht_dense_per_sm_f32 : dev.ht_dense_per_sm_bf16;
-    const int per_chunk = sizeof(GT) == 4 ? dev.ht_stream_per_sm_f32 : dev.ht_stream_per_sm_bf16;
-    if (use_group_kernel(tiles)) {
-      const int mode = stream_kernel_mode();
-      const bool dense =
-          mode == 3 || (mode == 0 && ws.density_host &&
-                        *static_cast<volatile uint32_t*>(ws.density_host) >= kDenseRingHint);
-      if (dense && per_dense > 0)
-        return launch_groups<GT, kHtStages<GT> - 1>(g, e, gamma, lambda, d, idx_out, val_out,
-                                                    count_out, err_out, tiles_out, ws, dev, ctx,
-                                                    per_dense);
-      if (per_group > 0)
-        return launch_groups<GT, kHtStages<GT>>(g, e, gamma, lambda, d, idx_out, val_out,
-                                                count_out, err_out, tiles_out, ws, dev, ctx,
-                                                per_group);
-    }
-    if (per_chunk > 0)
-      return launch_chunks(g, e, gamma, lambda, d, idx_out, val_out, count_out, err_out,
-                           tiles_out, ws, dev, ctx, per_chunk);
-  }
-  const bool vec = (ga % (4 * sizeof(GT)) == 0) && (ea % 16 == 0);
-  if (vec) {
-    ht_kernel<GT, true><<<tiles, kThreads, 0, ws.stream>>>(g, e, gamma, lambda, d, idx_out,
-                                                           val_out, count_out, ctx);
-  } else {
-    ht_kernel<GT, false><<<tiles, kThreads, 0, ws.stream>>>(g, e, gamma, lambda, d, idx_out,
-                                                            val_out, count_out, ctx);
-  }
-  count_launch();
-  cudaError_t err = cudaGetLastError();
-  if (err == cudaSuccess && err_out) err = launch_error_norm(e, d, err_out, ws, dev);
-  if (err == cudaSuccess && tiles_out) err = launch_list_tiles(idx_out, count_out, d, tiles_out, ws);
+  // the kernels' tile index is that of positions: with a shift, the message's
+  // comes from its list instead
+  uint32_t* kernel_tiles = in.shift_ == 0 ? tiles_out : nullptr;
+  const int per_group = sizeof(GT) == 4 ? dev.ht_group_per_sm_f32 : dev.ht_group_per_sm_bf16;
+  const int per_dense = sizeof(GT) == 4 ? dev.ht_dense_per_sm_f32 : dev.ht_dense_per_sm_bf16;
+  const int per_chunk = sizeof(GT) == 4 ? dev.ht_stream_per_sm_f32 : dev.ht_stream_per_sm_bf16;
+  cudaError_t err = cudaErrorInvalidConfiguration;
+  const int mode = stream_kernel_mode();
+  const bool groups = use_group_kernel(tiles) && per_group > 0;
+  const bool dense =
+      groups && per_dense > 0 &&
+      (mode == 3 || (mode == 0 && ws.density_host &&
+                     *static_cast<volatile uint32_t*>(ws.density_host) >= kDenseRingHint));
+  if (dense)
+    err = launch_groups<kHtStages<GT> - 1>(in, gamma, lambda, d, idx_out, val_out, count_out,
+                                               err_out, kernel_tiles, ws, dev, ctx, per_dense);
+  else if (groups)
+    err = launch_groups<kHtStages<GT>>(in, gamma, lambda, d, idx_out, val_out, count_out,
+                                           err_out, kernel_tiles, ws, dev, ctx, per_group);
+  else if (per_chunk > 0)
+    err = launch_chunks(in, gamma, lambda, d, idx_out, val_out, count_out, err_out, kernel_tiles,
+                        ws, dev, ctx, per_chunk);
+  if (err == cudaSuccess && tiles_out && !kernel_tiles)
+    err = launch_list_tiles(idx_out, count_out, d, tiles_out, ws);
   return err;
 }
 
@@ -326,16 +292,24 @@ int blocks_per_sm(const void* fn, int threads) {
   return n;
 }
 
+template <typename GT, bool kAny, int kStages>
+int group_blocks() {
+  return blocks_per_sm<GT, HtGroupKernel<GT, kAny, kStages>>(
+      reinterpret_cast<const void*>(&lookback_stream_kernel<HtOp<GT, kAny>, kStages>), kLbThreads);
+}
 template <typename GT, int kStages>
 int group_blocks_per_sm() {
-  return blocks_per_sm<GT, HtGroupKernel<GT, kStages>>(
-      reinterpret_cast<const void*>(&lookback_stream_kernel<HtOp<GT>, kStages>), kLbThreads);
+  return std::min(group_blocks<GT, false, kStages>(), group_blocks<GT, true, kStages>());
+}
+template <typename GT, bool kAny>
+int chunk_blocks() {
+  return blocks_per_sm<GT, HtChunkKernel<GT, kAny>>(
+      reinterpret_cast<const void*>(&stream_compact_kernel<HtOp<GT, kAny>, kHtStages<GT>>),
+      kStreamThreads);
 }
 template <typename GT>
 int chunk_blocks_per_sm() {
-  return blocks_per_sm<GT, HtChunkKernel<GT>>(
-      reinterpret_cast<const void*>(&stream_compact_kernel<HtOp<GT>, kHtStages<GT>>),
-      kStreamThreads);
+  return std::min(chunk_blocks<GT, false>(), chunk_blocks<GT, true>());
 }
 
 }  // namespace
@@ -359,10 +333,10 @@ cudaError_t launch_hard_threshold_lookback(const float* g, float* e, float gamma
   const bool vec = reinterpret_cast<uintptr_t>(g) % 16 == 0 &&
                    reinterpret_cast<uintptr_t>(e) % 16 == 0;
   if (vec)
-    ht_kernel<float, true><<<tiles, kThreads, 0, stream>>>(g, e, gamma, lambda, d, idx_out,
+    ht_kernel<true><<<tiles, kThreads, 0, stream>>>(g, e, gamma, lambda, d, idx_out,
                                                            val_out, count_out, ctx);
   else
-    ht_kernel<float, false><<<tiles, kThreads, 0, stream>>>(g, e, gamma, lambda, d, idx_out,
+    ht_kernel<false><<<tiles, kThreads, 0, stream>>>(g, e, gamma, lambda, d, idx_out,
                                                             val_out, count_out, ctx);
   count_launch();
   return cudaGetLastError();
@@ -372,11 +346,14 @@ cudaError_t launch_hard_threshold(const void* g, bool g_bf16, float* e, float ga
                                   float lambda, uint32_t d, uint32_t* idx_out, float* val_out,
                                   uint32_t* count_out, double* err_out, uint32_t* tiles_out,
                                   Workspace& ws, const DeviceInfo& dev) {
-  if (g_bf16)
-    return launch_typed(static_cast<const uint16_t*>(g), e, gamma, lambda, d, idx_out, val_out,
-                        count_out, err_out, tiles_out, ws, dev);
-  return launch_typed(static_cast<const float*>(g), e, gamma, lambda, d, idx_out, val_out,
-                      count_out, err_out, tiles_out, ws, dev);
+  auto run = [&](auto* gt) {
+    return positions(gt, e).any()
+               ? launch_typed<true>(gt, e, gamma, lambda, d, idx_out, val_out, count_out, err_out,
+                                    tiles_out, ws, dev)
+               : launch_typed<false>(gt, e, gamma, lambda, d, idx_out, val_out, count_out,
+                                     err_out, tiles_out, ws, dev);
+  };
+  return g_bf16 ? run(static_cast<const uint16_t*>(g)) : run(static_cast<const float*>(g));
 }
 
 }  // namespace efs

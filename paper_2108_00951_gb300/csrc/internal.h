@@ -229,11 +229,6 @@ cudaError_t launch_scaled_round(const void* g, bool g_bf16, float* e, float gamm
 cudaError_t launch_int_aggregate(uint32_t n, const int32_t* const* q, uint32_t d, int m,
                                  float* dense_out, Workspace& ws, const DeviceInfo& dev);
 
-// ||e'||^2 of e[0, d) after a step, by one plain pass (the paths that do
-// not stream through stream_compact.cuh); written to *err_out.
-cudaError_t launch_error_norm(const float* e, uint32_t d, double* err_out, Workspace& ws,
-                              const DeviceInfo& dev);
-
 // Launch bookkeeping.
 // A launch that may begin while the previous kernel on the stream finishes
 // (programmatic dependent launch: the kernel waits for its predecessor with
@@ -273,8 +268,8 @@ cudaError_t launch_hard_threshold(const void* g, bool g_bf16, float* e, float ga
                                   float lambda, uint32_t d, uint32_t* idx_out, float* val_out,
                                   uint32_t* count_out, double* err_out, uint32_t* tiles_out,
                                   Workspace& ws, const DeviceInfo& dev);
-// The tile index of one ascending list (binary searches), for the paths whose
-// kernel does not produce it.
+// The tile index of one ascending list (agg_offsets_kernel), for the calls
+// whose kernel does not produce it.
 cudaError_t launch_list_tiles(const uint32_t* idx, const uint32_t* count, uint32_t d,
                               uint32_t* tiles_out, Workspace& ws);
 cudaError_t launch_hard_threshold_lookback(const float* g, float* e, float gamma, float lambda,
@@ -306,6 +301,9 @@ cudaError_t launch_aggregate_apply(uint32_t n, const uint32_t* const* idx,
 inline uint32_t tiles_for(uint64_t d) {
   return static_cast<uint32_t>((d + kTileElems - 1) / kTileElems);
 }
+// Tiles of a streaming pass at any alignment of its inputs: they may start up
+// to 7 coordinates into the first tile (stream_in.cuh).
+inline uint32_t stream_tiles_for(uint64_t d) { return tiles_for(d + 7); }
 constexpr int kAggTile = 4096;             // dense elements per aggregation CTA
 constexpr int kAggStage = 1024;            // pairs an aggregation CTA stages per round trip
 static_assert(kAggTile == kTileElems, "a message's tile index serves the aggregation");

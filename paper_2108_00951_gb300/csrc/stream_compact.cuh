@@ -46,16 +46,19 @@
 // release, an earlier chunk's total) is bounded and latches kDevErrTimeout;
 // after a timeout the CTA places no pair.
 //
-// An Op supplies the per-segment work:
+// An Op supplies the per-segment work (on positions: coordinates plus
+// op.shift(); its inputs, from which it takes shift(), full(), fill(), prefetch()
+// and kStageBytes, are a StreamIn, stream_in.cuh):
 //   static constexpr uint32_t kStageBytes;            bytes of one stage
+//   bool full(uint32_t tile)                          every position is a coordinate
 //   void fill(unsigned char* stage, uint32_t tile, uint64_t* bar, uint64_t pol)
-//        issue the bulk copies of a full tile (after expect_tx)
+//        announce and issue the bulk copies of a full tile
 //   void tile_smem(const unsigned char* stage, uint32_t tile, int warp, int lane,
 //                  float (&a)[kSUnits][4], uint32_t (&sel)[kSUnits])
 //   void tile_global(uint32_t tile, int warp, int lane, float (&a)[..], uint32_t (&sel)[..])
 //        compute values and selection bits (and side effects) of the calling
 //        warp's segment, from the stage of a full tile, or from global memory
-//        for the partial last tile.
+//        for a partial one (the last, and the first when shift() > 0).
 //   (tile_smem and tile_global also receive `aux`, from
 //   uint64_t initial_aux()  (all threads, after the wait for the previous
 //   kernel; uniform))
@@ -64,12 +67,12 @@
 //   void prefetch(uint32_t tile)               L2 before the wait for the previous kernel
 //   static constexpr bool kKeepPairs;  the pairs are written with the L2
 //                                      evict-last policy (a later kernel of the call reads them)
-// Element layout: unit v of lane l of warp w covers the 4 coordinates from
+// Element layout: unit v of lane l of warp w covers the 4 positions from
 // tile * kTileElems + w * 256 + v * 128 + l * 4 (see stream_element_index).
 #pragma once
 
 #include "compact.cuh"
-#include "tma.cuh"
+#include "stream_in.cuh"
 
 namespace efs {
 
@@ -191,13 +194,12 @@ struct StreamLayout {
   static constexpr uint32_t kSmem = kRing + kStaging;  // dynamic shared memory
   // phase 2 reuses the ring: per segment of a window, its output offset and
   // its warp's count of earlier pairs in the chunk
-  static constexpr uint32_t kChunkSegs = kRing / 8;
-  static_assert(kChunkSegs % kSWarps == 0, "whole tiles per window");
+  static constexpr uint32_t kChunkSegs = kRing / 8 / kSWarps * kSWarps;  // whole tiles
 };
 
 template <class Op, int kStages>
 __global__ void __launch_bounds__(kStreamThreads, 1)
-    stream_compact_kernel(Op op, uint32_t d, uint32_t* __restrict__ idx_out,
+    stream_compact_kernel(Op op, uint32_t* __restrict__ idx_out,
                           float* __restrict__ val_out, uint32_t* __restrict__ count_out,
                           uint32_t cap, ScanCtx ctx, StreamArgs sa) {
   extern __shared__ __align__(128) unsigned char smem[];
@@ -220,7 +222,6 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
     t_hi = min(max(__ldcg(sa.part_in + c + 1), t_lo), T);
   }
   const uint32_t rounds = t_hi - t_lo;
-  const uint32_t full_tiles = d / kTileElems;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 
   if (threadIdx.x == 0) {
@@ -238,7 +239,7 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
   // bulk copies below read these lines.
   if (threadIdx.x == 0)
     for (uint32_t r = 0; r < rounds && r < Op::kPrefetchTiles; ++r)
-      if (t_lo + r < full_tiles) op.prefetch(t_lo + r);
+      if (op.full(t_lo + r)) op.prefetch(t_lo + r);
   // everything the previous kernels on the stream wrote is read only after this
   griddep_wait();
   op.prologue();
@@ -252,12 +253,10 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
   auto fill = [&](uint32_t r) {  // producer lane
     const int s = static_cast<int>(r % kStages);
     const uint32_t t = t_lo + r;
-    if (t < full_tiles) {
-      mbar_arrive_expect_tx(&s_full[s], Op::kStageBytes);
+    if (op.full(t))
       op.fill(smem + s * Op::kStageBytes, t, &s_full[s], policy);
-    } else {
-      mbar_arrive(&s_full[s]);  // the partial last tile is read from global memory
-    }
+    else
+      mbar_arrive(&s_full[s]);  // a partial tile is read from global memory
   };
   const bool producer = warp == kProducerWarp && lane == 0;
   if (producer) {
@@ -309,7 +308,7 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
       }
       float a[kSUnits][4];
       uint32_t sel[kSUnits];
-      if (t < full_tiles) {
+      if (op.full(t)) {
         op.tile_smem(smem + s * Op::kStageBytes, t, warp, lane, a, sel, aux);
       } else {
         op.tile_global(t, warp, lane, a, sel, aux);
@@ -357,7 +356,8 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
 #pragma unroll
           for (int j = 0; j < 4; ++j) {
             if (sel[v] & (1u << j)) {
-              sidx[pos] = static_cast<uint32_t>(stream_element_index(t, warp, v, lane, j));
+              sidx[pos] =
+                  static_cast<uint32_t>(stream_element_index(t, warp, v, lane, j)) - op.shift();
               sval[pos] = a[v][j];
               ++pos;
             }

@@ -186,7 +186,7 @@ __device__ __forceinline__ bool lb_withheld(const ScanCtx& ctx, uint32_t group) 
 
 template <class Op, int kStages>
 __global__ void __launch_bounds__(kLbThreads, 1)
-    lookback_stream_kernel(Op op, uint32_t d, uint32_t* __restrict__ idx_out,
+    lookback_stream_kernel(Op op, uint32_t* __restrict__ idx_out,
                            float* __restrict__ val_out, uint32_t* __restrict__ count_out,
                            uint32_t cap, ScanCtx ctx, LbArgs la) {
   extern __shared__ __align__(128) unsigned char smem[];
@@ -211,7 +211,6 @@ __global__ void __launch_bounds__(kLbThreads, 1)
 
   const uint32_t T = ctx.num_tiles;
   const uint32_t G = (T + kLbGroupTiles - 1) / kLbGroupTiles;
-  const uint32_t full_tiles = d / kTileElems;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 
   if (threadIdx.x == 0) {
@@ -240,11 +239,10 @@ __global__ void __launch_bounds__(kLbThreads, 1)
   // coherence, so the previous kernel's writes still land before the bulk
   // copies read these lines. Whole tiles only.
   if (threadIdx.x == 0 && Op::kPrefetchTiles > 0) {
-    const uint32_t full_tiles = d / kTileElems;
     for (uint32_t r = 0; r < 2; ++r)
       for (uint32_t j = 0; j < kLbGroupTiles; ++j) {
         const uint32_t t = (blockIdx.x + r * gridDim.x) * kLbGroupTiles + j;
-        if (t < full_tiles) op.prefetch(t);
+        if (op.full(t)) op.prefetch(t);
       }
   }
   // everything the previous kernels on the stream wrote (and the reset
@@ -313,12 +311,10 @@ __global__ void __launch_bounds__(kLbThreads, 1)
           const uint32_t t = g * kLbGroupTiles + q;
           s_stage_tile[s] = t;
           s_stage_info[s] = slot | (q << 8);
-          if (t < full_tiles) {
-            mbar_arrive_expect_tx(&s_full[s], Op::kStageBytes);
+          if (op.full(t))
             op.fill(smem + s * Op::kStageBytes, t, &s_full[s], policy);
-          } else {
-            mbar_arrive(&s_full[s]);  // the partial last tile is read from global memory
-          }
+          else
+            mbar_arrive(&s_full[s]);  // a partial tile is read from global memory
         }
         ++seq;
       }
@@ -400,7 +396,8 @@ __global__ void __launch_bounds__(kLbThreads, 1)
           *count_out = end < cap ? end : cap;
           if (la.tile_base) la.tile_base[T] = end;
           if (la.density_out)
-            *la.density_out = static_cast<uint32_t>((static_cast<uint64_t>(end) << 16) / d);
+            *la.density_out =
+                static_cast<uint32_t>((static_cast<uint64_t>(end) << 16) / (op.end - op.shift()));
         }
         if (la.err_out) {
           FF s{0.0f, 0.0f};
@@ -454,14 +451,14 @@ __global__ void __launch_bounds__(kLbThreads, 1)
       const int w = lane & (kSWarps - 1);
       // a buffered segment's first pair: its warp's head, after the warp's
       // tile-0 segment when that one is buffered too (kLbGroupTiles == 2); a
-      // slotted segment's: its slot
+      // slotted segment's: its slot's number
       uint32_t src = __shfl_sync(0xffffffffu, head, w);
       const uint32_t c_prev = __shfl_sync(0xffffffffu, c_buf, (lane - kSWarps) & 31);
       if (lane >= kSWarps) src += c_prev;
       if (src >= L::kFifo) src -= L::kFifo;
       if (in_slot)
-        src = ((en.group * kLbGroupTiles + static_cast<uint32_t>(lane) / kSWarps) * kSWarps +
-               static_cast<uint32_t>(w)) * static_cast<uint32_t>(kSWarpElems);
+        src = (en.group * kLbGroupTiles + static_cast<uint32_t>(lane) / kSWarps) * kSWarps +
+              static_cast<uint32_t>(w);
       // placer warp p copies the segments l = p, p + kLbPlaceWarps, ...: the
       // segment's pairs are consecutive in its source and in the output, so
       // the warp's lanes take consecutive pairs (coalesced loads and stores)
@@ -475,7 +472,7 @@ __global__ void __launch_bounds__(kLbThreads, 1)
           uint32_t xi;
           float xv;
           if (slotted) {
-            const size_t b = static_cast<size_t>(sl) + k;
+            const size_t b = static_cast<size_t>(sl) * kSWarpElems + k;
             xi = la.slot_idx[b];  // written by a warp of this CTA (ordered by the fences)
             xv = la.slot_val[b];
           } else {
@@ -527,7 +524,7 @@ __global__ void __launch_bounds__(kLbThreads, 1)
     // buffer, counts, arrival) is done once for both tiles.
     auto compute_tile = [&](int s, uint32_t t, float (&a)[kSUnits][4],
                             uint32_t (&sel)[kSUnits]) {
-      if (t < full_tiles) {
+      if (op.full(t)) {
         op.tile_smem(smem + s * Op::kStageBytes, t, warp, lane, a, sel, aux);
       } else {
         op.tile_global(t, warp, lane, a, sel, aux);
@@ -608,7 +605,7 @@ __global__ void __launch_bounds__(kLbThreads, 1)
       for (int q = 0; q < 2; ++q) {
         const uint32_t t = t0 + q;
         const uint32_t first_elem =
-            static_cast<uint32_t>(stream_element_index(t, warp, 0, lane, 0));
+            static_cast<uint32_t>(stream_element_index(t, warp, 0, lane, 0)) - op.shift();
         if ((to_slot >> q) & 1u) {
           const size_t sb = (static_cast<size_t>(t) * kSWarps + warp) * kSWarpElems;
 #pragma unroll

@@ -34,7 +34,8 @@
 //             positions).
 // The candidate path moves about 12 B per coordinate plus small amounts; the
 // full-array path adds a read of a per digit level and two for the output.
-#include "gradient.cuh"
+#include <algorithm>
+
 #include "internal.h"
 #include "select.cuh"
 #include "stream_lookback.cuh"
@@ -87,10 +88,8 @@ struct TopkArgs {
 // chooses the full-array mode (nothing gathered). Streaming: a = fmaf(γ,g,e)
 // is written over e and the coordinates with K_j >= B are selected (ordered
 // candidates).
-template <typename GT>
-struct TopkCandOp {
-  const GT* g;
-  float* e;
+template <typename GT, bool kAny>
+struct TopkCandOp : StreamIn<GT, kAny> {
   float gamma;
   uint32_t d, k, cand_cap;
   uint32_t* hist;      // global sample histogram [kSampleBins]
@@ -98,8 +97,6 @@ struct TopkCandOp {
   uint32_t* mode;      // published for the select kernel
   uint64_t* lower_bound;
   uint32_t* other_state;    // the other state block: zeroed here for the next call
-  static constexpr uint32_t kGBytes = kTileElems * sizeof(GT);
-  static constexpr uint32_t kStageBytes = kGBytes + kTileElems * sizeof(float);
   static constexpr uint32_t kWarpStagePairs = 512;  // on-chip staged pairs per compute warp
   static constexpr bool kKeepPairs = true;  // the candidate list: the select reads it next
   static constexpr int kSampleBins = efs::kSampleBins;
@@ -108,56 +105,24 @@ struct TopkCandOp {
   // no L2 prefetch before the wait: measured 3 %% slower (the previous call's
   // select, still running, re-reads its candidate list from L2)
   static constexpr uint32_t kPrefetchTiles = 0;
-  __device__ __forceinline__ void prefetch(uint32_t t) const {
-    prefetch_l2_1d(g + static_cast<size_t>(t) * kTileElems, kGBytes);
-    prefetch_l2_1d(e + static_cast<size_t>(t) * kTileElems, kTileElems * sizeof(float));
-  }
-  __device__ __forceinline__ void fill(unsigned char* stage, uint32_t t, uint64_t* bar,
-                                       uint64_t policy) const {
-    tma_load_1d(stage, g + static_cast<size_t>(t) * kTileElems, kGBytes, bar, policy);
-    tma_load_1d(stage + kGBytes, e + static_cast<size_t>(t) * kTileElems,
-                kTileElems * sizeof(float), bar, policy);
-  }
 
-  __device__ __forceinline__ void accumulate(const unsigned char* stage, int warp, int lane, int v,
-                                             float (&x)[4]) const {
-    const GT* gs = reinterpret_cast<const GT*>(stage);
-    const float* es = reinterpret_cast<const float*>(stage + kGBytes);
-    const int local = warp * kSWarpElems + lane * 4 + v * 128;
-    GradVec<GT> gv;
-    if constexpr (sizeof(GT) == 4)
-      gv.v = *reinterpret_cast<const float4*>(gs + local);
-    else
-      gv.v = *reinterpret_cast<const uint2*>(gs + local);
-    const float4 ev = *reinterpret_cast<const float4*>(es + local);
-    x[0] = __fmaf_rn(gamma, gv[0], ev.x);
-    x[1] = __fmaf_rn(gamma, gv[1], ev.y);
-    x[2] = __fmaf_rn(gamma, gv[2], ev.z);
-    x[3] = __fmaf_rn(gamma, gv[3], ev.w);
-  }
-
-  // The sample: each compute thread reads one aligned group of 4 coordinates
+  // The sample: each compute thread reads one aligned group of 4 positions
   // of g and e straight from global memory (issued together with the ring's
   // first fills), the groups spread evenly over the CTA's chunk.
   __device__ void sample(uint32_t t_lo, uint32_t t_hi, int tid, uint32_t* s_hist) const {
-    const uint64_t lo = static_cast<uint64_t>(t_lo) * kTileElems;
-    const uint64_t end = static_cast<uint64_t>(t_hi) * kTileElems;
-    const uint64_t hi = end < d ? end : d;
-    const uint64_t groups = (hi - lo) / 4;  // whole groups of 4 inside [lo, hi)
+    const uint64_t first = (static_cast<uint64_t>(this->shift()) + 3) & ~static_cast<uint64_t>(3);
+    const uint64_t lo = t_lo == 0 ? first : static_cast<uint64_t>(t_lo) * kTileElems;
+    const uint64_t stop = static_cast<uint64_t>(t_hi) * kTileElems;
+    const uint64_t hi = stop < this->end ? stop : this->end;
+    // whole groups of 4 inside [lo, hi)
+    const uint64_t groups = hi > lo ? (hi - lo) / 4 : 0;
     const uint64_t grp = groups >= static_cast<uint64_t>(kComputeThreads)
                              ? static_cast<uint64_t>(tid) * groups / kComputeThreads
                              : static_cast<uint64_t>(tid);
     const bool in = grp < groups;
     GradVec<GT> gv;
     float4 ev = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-    if (in) {
-      const uint64_t p = lo + grp * 4;
-      if constexpr (sizeof(GT) == 4)
-        gv.v = __ldg(reinterpret_cast<const float4*>(g + p));
-      else
-        gv.v = __ldg(reinterpret_cast<const uint2*>(g + p));
-      ev = __ldg(reinterpret_cast<const float4*>(e + p));
-    }
+    if (in) this->load4(lo + grp * 4, gv, ev);
     float x[4] = {0.0f, 0.0f, 0.0f, 0.0f};
     if (in) {
       x[0] = __fmaf_rn(gamma, gv[0], ev.x);
@@ -284,14 +249,15 @@ struct TopkCandOp {
                                             int lane, float (&a)[kSUnits][4],
                                             uint32_t (&sel)[kSUnits], uint64_t bound) const {
     const uint64_t first = stream_element_index(t, warp, 0, lane, 0);
+    const uint32_t least = bound_magnitude(bound);
 #pragma unroll
     for (int v = 0; v < kSUnits; ++v) {
-      accumulate(stage, warp, lane, v, a[v]);
-      st_stream_f4(e + first + v * 128, make_float4(a[v][0], a[v][1], a[v][2], a[v][3]));
+      this->accumulate(stage, warp * kSWarpElems + lane * 4 + v * 128, gamma, a[v]);
+      st_stream_f4(this->e + first + v * 128, make_float4(a[v][0], a[v][1], a[v][2], a[v][3]));
       sel[v] = 0;
 #pragma unroll
       for (int j = 0; j < 4; ++j)
-        sel[v] |= (composite_key(a[v][j], first + v * 128 + j) >= bound ? 1u : 0u) << j;
+        sel[v] |= ((__float_as_uint(a[v][j]) & 0x7fffffffu) >= least ? 1u : 0u) << j;
     }
   }
 
@@ -299,6 +265,7 @@ struct TopkCandOp {
                                               float (&a)[kSUnits][4],
                                               uint32_t (&sel)[kSUnits], uint64_t bound) const {
     const uint64_t first = stream_element_index(t, warp, 0, lane, 0);
+    const uint32_t least = bound_magnitude(bound);
 #pragma unroll
     for (int v = 0; v < kSUnits; ++v) {
       sel[v] = 0;
@@ -306,14 +273,20 @@ struct TopkCandOp {
       for (int j = 0; j < 4; ++j) {
         const uint64_t i = first + v * 128 + j;
         a[v][j] = 0.0f;
-        if (i < d) {
-          const float x = __fmaf_rn(gamma, grad_scalar(g, i), e[i]);
-          e[i] = x;
+        if (this->valid(i)) {
+          const float x = this->accumulate_at(i, gamma);
+          this->e[i] = x;
           a[v][j] = x;
-          sel[v] |= (composite_key(x, i) >= bound ? 1u : 0u) << j;
+          sel[v] |= ((__float_as_uint(x) & 0x7fffffffu) >= least ? 1u : 0u) << j;
         }
       }
     }
+  }
+
+  // A bound is a bin's lower edge (or kSelectNone): its index part is zero,
+  // so K_j >= bound is a comparison of the magnitude bits alone.
+  static __device__ __forceinline__ uint32_t bound_magnitude(uint64_t bound) {
+    return static_cast<uint32_t>(bound >> 32);
   }
 };
 
@@ -336,14 +309,14 @@ constexpr int kTkStages = 4;
 // for it before letting this kernel start). Only the last CTA waits, so the
 // grid completes after the previous kernel; the others leave their SMs to the
 // streaming pass, which may be scheduled from the start.
-template <typename GT>
+template <typename GT, bool kAny>
 __global__ void __launch_bounds__(kStreamThreads)
-    topk_sample_kernel(TopkCandOp<GT> op, uint32_t num_tiles) {
-  __shared__ uint32_t s_hist[TopkCandOp<GT>::kSampleBins];
+    topk_sample_kernel(TopkCandOp<GT, kAny> op, uint32_t num_tiles) {
+  __shared__ uint32_t s_hist[TopkCandOp<GT, kAny>::kSampleBins];
   const uint32_t T = num_tiles, G = gridDim.x, c = blockIdx.x;
   const uint32_t t_lo = static_cast<uint32_t>(static_cast<uint64_t>(c) * T / G);
   const uint32_t t_hi = static_cast<uint32_t>(static_cast<uint64_t>(c + 1) * T / G);
-  for (int b = threadIdx.x; b < TopkCandOp<GT>::kSampleBins; b += blockDim.x) s_hist[b] = 0;
+  for (int b = threadIdx.x; b < TopkCandOp<GT, kAny>::kSampleBins; b += blockDim.x) s_hist[b] = 0;
   griddep_launch_dependents();  // the streaming pass waits for this whole grid
   __syncthreads();
   if (threadIdx.x < kComputeThreads && t_hi > t_lo) op.sample(t_lo, t_hi, threadIdx.x, s_hist);
@@ -352,23 +325,6 @@ __global__ void __launch_bounds__(kStreamThreads)
   if (!op.arrive_last()) return;
   op.choose();
   griddep_wait();  // this grid completes after the previous kernel
-}
-
-// Inputs the bulk copies cannot take (not 16-byte aligned): a = fmaf(γ,g,e)
-// written over e with plain loads, and the selection switched to the
-// full-array mode (block 0 runs after the sampling kernel on the stream).
-template <typename GT>
-__global__ void __launch_bounds__(kThreads)
-    topk_accumulate_plain_kernel(const GT* __restrict__ g, float* __restrict__ e, float gamma,
-                                 uint32_t d, TopkArgs args, uint32_t* other_state) {
-  clear_state(other_state);
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    *args.mode = 1;
-    *args.lower_bound = kSelectNone;
-  }
-  for (uint64_t i = static_cast<uint64_t>(blockIdx.x) * kThreads + threadIdx.x; i < d;
-       i += static_cast<uint64_t>(gridDim.x) * kThreads)
-    e[i] = __fmaf_rn(gamma, grad_scalar(g, i), e[i]);
 }
 
 // Reads the (mode, source length) a refine/finalize launch works on; the
@@ -863,11 +819,11 @@ __global__ void __launch_bounds__(kSelThreads, 1)
   if (__syncthreads_or(overflow) && threadIdx.x == 0) atomicOr(args.error, kDevErrOverflow);
 }
 
-template <typename GT>
+template <typename GT, bool kAny>
 int tk_group_blocks_per_sm() {
   const void* fn =
-      reinterpret_cast<const void*>(&lookback_stream_kernel<TopkCandOp<GT>, kTkStages>);
-  const uint32_t smem = LbLayout<TopkCandOp<GT>, kTkStages>::kSmem;
+      reinterpret_cast<const void*>(&lookback_stream_kernel<TopkCandOp<GT, kAny>, kTkStages>);
+  const uint32_t smem = LbLayout<TopkCandOp<GT, kAny>, kTkStages>::kSmem;
   int n = 0;
   if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fn, kLbThreads, smem) != cudaSuccess)
@@ -876,10 +832,10 @@ int tk_group_blocks_per_sm() {
   return n;
 }
 
-template <typename GT>
+template <typename GT, bool kAny>
 int tk_stream_blocks_per_sm() {
-  const void* fn = reinterpret_cast<const void*>(&stream_compact_kernel<TopkCandOp<GT>, kTkStages>);
-  const uint32_t smem = StreamLayout<TopkCandOp<GT>, kTkStages>::kSmem;
+  const void* fn = reinterpret_cast<const void*>(&stream_compact_kernel<TopkCandOp<GT, kAny>, kTkStages>);
+  const uint32_t smem = StreamLayout<TopkCandOp<GT, kAny>, kTkStages>::kSmem;
   int n = 0;
   if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fn, kStreamThreads, smem) != cudaSuccess)
@@ -888,11 +844,12 @@ int tk_stream_blocks_per_sm() {
   return n;
 }
 
-template <typename GT>
+template <bool kAny, typename GT>
 cudaError_t launch_typed(const GT* g, float* e, float gamma, uint32_t k, uint32_t d,
                          uint32_t* idx_out, float* val_out, uint32_t* count_out, double* err_out,
                          Workspace& ws, const DeviceInfo& dev) {
-  const uint32_t tiles = tiles_for(d);
+  const StreamIn<GT, kAny> in = stream_in<GT, kAny>(g, e, d);
+  const uint32_t tiles = tiles_for(in.end);
   cudaError_t err = cudaSuccess;
   // this call's zeroed state block, and the other one, cleared for the next call
   uint32_t* state = ws.topk_state(ws.topk_calls);
@@ -921,64 +878,51 @@ cudaError_t launch_typed(const GT* g, float* e, float gamma, uint32_t k, uint32_
   args.stream_err = ws.stream_err();
   args.err_parts = ws.errparts();
 
-  // 1 sample + 2 stream (candidates). The bulk copies need 16-byte
-  // aligned g and e; otherwise a plain pass writes a and the selection runs in
-  // the full-array mode.
+  // 1 sample + 2 stream (candidates)
   ScanCtx ctx = next_scan_ctx(ws, tiles);
   ctx.error = args.list_flags;
   const int per_sm = sizeof(GT) == 4 ? dev.tk_stream_per_sm_f32 : dev.tk_stream_per_sm_bf16;
   const int per_sm_groups =
       sizeof(GT) == 4 ? dev.tk_group_per_sm_f32 : dev.tk_group_per_sm_bf16;
-  const bool streamable = reinterpret_cast<uintptr_t>(e) % 16 == 0 &&
-                          reinterpret_cast<uintptr_t>(g) % 16 == 0 && per_sm > 0;
-  if (streamable) {
-    TopkCandOp<GT> op{g, e, gamma, d, k, ws.cand_cap, state + kStSampleHist / 4,
-                      state + kStStreamArrive / 4, args.mode, args.lower_bound, other};
-    uint32_t slots = static_cast<uint32_t>(per_sm * dev.sm_count);
-    if (slots > kMaxChunks) slots = kMaxChunks;
-    const uint32_t grid = tiles < slots ? tiles : slots;
-    uint32_t cap = ws.cand_cap;
+  if (per_sm <= 0) return cudaErrorInvalidConfiguration;
+  TopkCandOp<GT, kAny> op{in, gamma, d, k, ws.cand_cap, state + kStSampleHist / 4,
+                    state + kStStreamArrive / 4, args.mode, args.lower_bound, other};
+  uint32_t slots = static_cast<uint32_t>(per_sm * dev.sm_count);
+  if (slots > kMaxChunks) slots = kMaxChunks;
+  const uint32_t stream_grid = tiles < slots ? tiles : slots;
+  uint32_t cap = ws.cand_cap;
+  // the bound first (a small kernel without waits), then the streaming
+  // pass, whose CTAs only wait for lower-numbered ones: plain launches
+  uint32_t tiles_arg = tiles;
+  void* sp[] = {&op, &tiles_arg};
+  err = launch_pdl(reinterpret_cast<const void*>(&topk_sample_kernel<GT, kAny>), stream_grid,
+                   kStreamThreads, 0, ws.stream, sp, false);
+  count_launch();
+  if (err != cudaSuccess) return err;
+  if (use_group_kernel(tiles) && per_sm_groups > 0) {
+    // claimed groups of tiles with look-back (stream_lookback.cuh): no
+    // wait depends on which CTAs are resident
+    const uint32_t groups = (tiles + kLbGroupTiles - 1) / kLbGroupTiles;
+    const uint32_t gslots = static_cast<uint32_t>(per_sm_groups * dev.sm_count);
+    const uint32_t ggrid = groups < gslots ? groups : gslots;
+    LbArgs la{nullptr, err_out ? ws.stream_err() : nullptr, reinterpret_cast<FF*>(ws.counts()),
+              ws.stage_idx(), ws.stage_val()};
+    void* gp[] = {&op, &args.list_idx, &args.list_val, &args.list_count, &cap, &ctx, &la};
+    err = launch_pdl(
+        reinterpret_cast<const void*>(&lookback_stream_kernel<TopkCandOp<GT, kAny>, kTkStages>), ggrid,
+        kLbThreads, LbLayout<TopkCandOp<GT, kAny>, kTkStages>::kSmem, ws.stream, gp, false);
+  } else {
     StreamArgs sa{ws.stage_idx(), ws.stage_val(), ws.counts(), ws.chunks(), nullptr,
                   err_out ? ws.stream_err() : nullptr, ws.errparts()};
-    void* params[] = {&op, &d, &args.list_idx, &args.list_val, &args.list_count, &cap, &ctx, &sa};
-    // the bound first (a small kernel without waits), then the streaming
-    // pass, whose CTAs only wait for lower-numbered ones: plain launches
-    uint32_t tiles_arg = tiles;
-    void* sp[] = {&op, &tiles_arg};
-    err = launch_pdl(reinterpret_cast<const void*>(&topk_sample_kernel<GT>), grid, kStreamThreads,
-                     0, ws.stream, sp, false);
-    count_launch();
-    if (err != cudaSuccess) return err;
-    if (use_group_kernel(tiles) && per_sm_groups > 0) {
-      // claimed groups of tiles with look-back (stream_lookback.cuh): no
-      // wait depends on which CTAs are resident
-      const uint32_t groups = (tiles + kLbGroupTiles - 1) / kLbGroupTiles;
-      const uint32_t gslots = static_cast<uint32_t>(per_sm_groups * dev.sm_count);
-      const uint32_t ggrid = groups < gslots ? groups : gslots;
-      LbArgs la{nullptr, err_out ? ws.stream_err() : nullptr, reinterpret_cast<FF*>(ws.counts()),
-                ws.stage_idx(), ws.stage_val()};
-      void* gp[] = {&op, &d, &args.list_idx, &args.list_val, &args.list_count, &cap, &ctx, &la};
-      err = launch_pdl(
-          reinterpret_cast<const void*>(&lookback_stream_kernel<TopkCandOp<GT>, kTkStages>),
-          ggrid, kLbThreads, LbLayout<TopkCandOp<GT>, kTkStages>::kSmem, ws.stream, gp, false);
-    } else {
-      err = launch_pdl(
-          reinterpret_cast<const void*>(&stream_compact_kernel<TopkCandOp<GT>, kTkStages>), grid,
-          kStreamThreads, StreamLayout<TopkCandOp<GT>, kTkStages>::kSmem, ws.stream, params,
-          false);
-    }
-    count_launch();
-    if (err != cudaSuccess) return err;
-  } else {
-    const uint32_t grid = tiles < static_cast<uint32_t>(dev.sm_count * 8)
-                              ? tiles : static_cast<uint32_t>(dev.sm_count * 8);
-    topk_accumulate_plain_kernel<GT><<<grid, kThreads, 0, ws.stream>>>(g, e, gamma, d, args,
-                                                                       other);
-    count_launch();
-    if ((err = cudaGetLastError()) != cudaSuccess) return err;
+    void* cp[] = {&op, &args.list_idx, &args.list_val, &args.list_count, &cap, &ctx, &sa};
+    err = launch_pdl(
+        reinterpret_cast<const void*>(&stream_compact_kernel<TopkCandOp<GT, kAny>, kTkStages>),
+        stream_grid, kStreamThreads, StreamLayout<TopkCandOp<GT, kAny>, kTkStages>::kSmem, ws.stream,
+        cp, false);
   }
-  // 3 select (inputs the streaming pass could not take: the norm by a plain pass after it)
-  if (!streamable) args.err_out = nullptr;
+  count_launch();
+  if (err != cudaSuccess) return err;
+  // 3 select
   args.epoch = next_scan_ctx(ws, 1).epoch;
   void* params[] = {(void*)&e, (void*)&d, (void*)&k, (void*)&idx_out, (void*)&val_out,
                     (void*)&count_out, (void*)&args};
@@ -988,7 +932,6 @@ cudaError_t launch_typed(const GT* g, float* e, float gamma, uint32_t k, uint32_
   err = launch_pdl(reinterpret_cast<const void*>(&topk_select_kernel), grid, kSelThreads,
                    kSelSmem, ws.stream, params, true);
   count_launch();
-  if (err == cudaSuccess && err_out && !streamable) err = launch_error_norm(e, d, err_out, ws, dev);
   return err;
 }
 
@@ -1000,10 +943,14 @@ void topk_init_device(DeviceInfo& info) {
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, topk_select_kernel, kSelThreads, kSelSmem);
   info.refine_blocks = a * info.sm_count;
   info.finalize_blocks = info.refine_blocks;
-  info.tk_stream_per_sm_f32 = tk_stream_blocks_per_sm<float>();
-  info.tk_stream_per_sm_bf16 = tk_stream_blocks_per_sm<uint16_t>();
-  info.tk_group_per_sm_f32 = tk_group_blocks_per_sm<float>();
-  info.tk_group_per_sm_bf16 = tk_group_blocks_per_sm<uint16_t>();
+  info.tk_stream_per_sm_f32 =
+      std::min(tk_stream_blocks_per_sm<float, false>(), tk_stream_blocks_per_sm<float, true>());
+  info.tk_stream_per_sm_bf16 =
+      std::min(tk_stream_blocks_per_sm<uint16_t, false>(), tk_stream_blocks_per_sm<uint16_t, true>());
+  info.tk_group_per_sm_f32 =
+      std::min(tk_group_blocks_per_sm<float, false>(), tk_group_blocks_per_sm<float, true>());
+  info.tk_group_per_sm_bf16 =
+      std::min(tk_group_blocks_per_sm<uint16_t, false>(), tk_group_blocks_per_sm<uint16_t, true>());
   cudaGetLastError();
 }
 
@@ -1018,11 +965,13 @@ uint32_t topk_candidate_capacity(uint64_t d) {
 cudaError_t launch_topk(const void* g, bool g_bf16, float* e, float gamma, uint32_t k,
                         uint32_t d, uint32_t* idx_out, float* val_out, uint32_t* count_out,
                         double* err_out, Workspace& ws, const DeviceInfo& dev) {
-  if (g_bf16)
-    return launch_typed(static_cast<const uint16_t*>(g), e, gamma, k, d, idx_out, val_out,
-                        count_out, err_out, ws, dev);
-  return launch_typed(static_cast<const float*>(g), e, gamma, k, d, idx_out, val_out, count_out,
-                      err_out, ws, dev);
+  auto run = [&](auto* gt) {
+    return positions(gt, e).any() ? launch_typed<true>(gt, e, gamma, k, d, idx_out, val_out,
+                                                       count_out, err_out, ws, dev)
+                                  : launch_typed<false>(gt, e, gamma, k, d, idx_out, val_out,
+                                                        count_out, err_out, ws, dev);
+  };
+  return g_bf16 ? run(static_cast<const uint16_t*>(g)) : run(static_cast<const float*>(g));
 }
 
 }  // namespace efs

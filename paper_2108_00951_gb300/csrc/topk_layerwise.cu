@@ -38,7 +38,6 @@
 #include <functional>
 #include <queue>
 
-#include "gradient.cuh"
 #include "internal.h"
 #include "select.cuh"
 #include "stream_lookback.cuh"
@@ -73,10 +72,10 @@ __device__ __forceinline__ uint32_t mag_bits(float x) { return __float_as_uint(x
 // sees the new one.
 constexpr int kSampleThreads = 1024;
 
-template <typename GT>
+template <typename GT, bool kAny>
 __global__ void __launch_bounds__(kSampleThreads, 1)
-    lw_sample_kernel(const GT* __restrict__ g, const float* __restrict__ e, float gamma,
-                     const LwSeg* __restrict__ segs, const uint2* __restrict__ sampled,
+    lw_sample_kernel(StreamIn<GT, kAny> src, float gamma, const LwSeg* __restrict__ segs,
+                     const uint2* __restrict__ sampled,
                      uint32_t* mbound, uint32_t cand_cap, uint32_t* part_hist) {
   extern __shared__ uint32_t s_hist[];  // [kLwSampleBins]
   __shared__ uint32_t s_w[kSampleThreads / 32];
@@ -90,14 +89,17 @@ __global__ void __launch_bounds__(kSampleThreads, 1)
                  slot = rec.y >> 16;
   LwSeg s = segs[si];
   for (uint32_t b = tid; b < kLwSampleBins; b += kSampleThreads) s_hist[b] = 0;
-  uint64_t a0 = (static_cast<uint64_t>(s.lo) + 3u) & ~static_cast<uint64_t>(3);
-  if (parts > 1) {
-    const uint64_t avail = (static_cast<uint64_t>(s.hi) - a0) / 4;  // whole groups inside
+  // positions from here on: the segment's [lo, hi) and its first multiple of 4
+  const uint64_t p_hi = static_cast<uint64_t>(s.hi) + src.shift();
+  uint64_t a0 = (static_cast<uint64_t>(s.lo) + src.shift() + 3u) & ~static_cast<uint64_t>(3);
+  if (parts > 1 || src.shift() != 0) {
+    // the host planned for one part of a vector without a shift: plan again
+    const uint64_t avail = (p_hi - a0) / 4;  // whole groups inside
     const uint64_t g0 = part * avail / parts, g1 = (part + 1) * avail / parts;
     const uint64_t n = g1 - g0;
     s.groups = static_cast<uint32_t>(n < kLwSampleGroups ? n : kLwSampleGroups);
     s.step = s.groups > 1 ? ((n - 1) << 32) / (s.groups - 1) : 0;
-    s.exact = 0;
+    s.exact = parts == 1 && s.groups == n;
     a0 += 4 * g0;
   }
   constexpr int kG = static_cast<int>(kLwSampleGroups / kSampleThreads);
@@ -109,13 +111,7 @@ __global__ void __launch_bounds__(kSampleThreads, 1)
     const uint32_t qq = q * kSampleThreads + tid;
     in[q] = qq < s.groups;
     const uint64_t p = a0 + 4u * ((static_cast<uint64_t>(in[q] ? qq : 0u) * s.step) >> 32);
-    if (in[q]) {
-      if constexpr (sizeof(GT) == 4)
-        gv[q].v = __ldg(reinterpret_cast<const float4*>(g + p));
-      else
-        gv[q].v = __ldg(reinterpret_cast<const uint2*>(g + p));
-      ev[q] = __ldg(reinterpret_cast<const float4*>(e + p));
-    }
+    if (in[q]) src.load4(p, gv[q], ev[q]);
   }
   __syncthreads();
 #pragma unroll
@@ -210,18 +206,14 @@ __global__ void __launch_bounds__(kSampleThreads, 1)
 // The streaming pass as a stream_compact op: a stage holds a tile of g then
 // the same tile of e; a is written over e from registers, and a coordinate
 // is a candidate when its magnitude bits reach its segment's bound.
-template <typename GT>
-struct LwCandOp {
-  const GT* g;
-  float* e;
+template <typename GT, bool kAny>
+struct LwCandOp : StreamIn<GT, kAny> {
   float gamma;
-  uint32_t d;
   const uint32_t* seg_end;    // [n_seg] exclusive segment ends
   const uint32_t* mbound;     // [n_seg] candidate bounds (kLwNoBound, kLwDeferred: none)
   const uint32_t* tile_info;  // [tiles] first segment of the tile | kLwTileUniform
+  uint32_t tiles;             // entries of tile_info
   uint32_t* other_state;      // the other Top-k state block: zeroed here for the next call
-  static constexpr uint32_t kGBytes = kTileElems * sizeof(GT);
-  static constexpr uint32_t kStageBytes = kGBytes + kTileElems * sizeof(float);
   static constexpr uint32_t kWarpStagePairs = 512;  // on-chip staged pairs per compute warp
   static constexpr bool kKeepPairs = true;  // the candidate list: the select reads it next
   __device__ void prologue() const { clear_state(other_state); }
@@ -230,22 +222,26 @@ struct LwCandOp {
   // the chunk's first tiles of g and e toward L2 before the wait for the
   // previous kernel (its tail leaves DRAM mostly idle)
   static constexpr uint32_t kPrefetchTiles = 8;
-  __device__ __forceinline__ void prefetch(uint32_t t) const {
-    prefetch_l2_1d(g + static_cast<size_t>(t) * kTileElems, kGBytes);
-    prefetch_l2_1d(e + static_cast<size_t>(t) * kTileElems, kTileElems * sizeof(float));
-  }
-  __device__ __forceinline__ void fill(unsigned char* stage, uint32_t t, uint64_t* bar,
-                                       uint64_t policy) const {
-    tma_load_1d(stage, g + static_cast<size_t>(t) * kTileElems, kGBytes, bar, policy);
-    tma_load_1d(stage + kGBytes, e + static_cast<size_t>(t) * kTileElems,
-                kTileElems * sizeof(float), bar, policy);
+
+  // The first segment of tile t of the positions, and whether the tile lies
+  // in it. tile_info is that of the coordinates: with a shift the tile starts
+  // up to 7 coordinates earlier, perhaps in an earlier segment.
+  __device__ __forceinline__ uint32_t segment_of_tile(uint32_t t) const {
+    if (this->shift() == 0) return __ldg(tile_info + t);
+    const uint64_t j0 = t == 0 ? 0 : static_cast<uint64_t>(t) * kTileElems - this->shift();
+    const uint64_t j1 = static_cast<uint64_t>(t + 1) * kTileElems - this->shift();
+    uint32_t s = __ldg(tile_info + min(t, tiles - 1)) & ~kLwTileUniform;
+    while (s > 0 && __ldg(seg_end + s - 1) > j0) --s;
+    while (__ldg(seg_end + s) <= j0) ++s;  // empty segments; seg_end[last] = d > j0
+    const uint64_t d = this->end - this->shift();
+    return s | (__ldg(seg_end + s) >= (j1 < d ? j1 : d) ? kLwTileUniform : 0u);
   }
 
   // selection bits of the lane's coordinates from their segments' bounds
   // (bit j: candidate; bit 4 + j: residual decided by the select)
   __device__ __forceinline__ void select(uint32_t t, uint64_t first, const float (&a)[kSUnits][4],
                                          uint32_t (&sel)[kSUnits]) const {
-    const uint32_t info = __ldg(tile_info + t);
+    const uint32_t info = segment_of_tile(t);
     if (info & kLwTileUniform) {
       const uint32_t b = __ldg(mbound + (info & ~kLwTileUniform));
       const uint32_t defer = b == kLwDeferred ? 0xf0u : 0u;
@@ -263,8 +259,8 @@ struct LwCandOp {
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
           const uint64_t i = first + v * 128 + j;
-          if (i < d) {
-            while (__ldg(seg_end + s) <= i) ++s;
+          if (this->valid(i)) {
+            while (__ldg(seg_end + s) <= i - this->shift()) ++s;
             const uint32_t b = __ldg(mbound + s);
             sel[v] |= (mag_bits(a[v][j]) >= b ? 1u : 0u) << j;
             sel[v] |= (b == kLwDeferred ? 1u : 0u) << (4 + j);
@@ -277,23 +273,11 @@ struct LwCandOp {
   __device__ __forceinline__ void tile_smem(const unsigned char* stage, uint32_t t, int warp,
                                             int lane, float (&a)[kSUnits][4],
                                             uint32_t (&sel)[kSUnits], uint64_t) const {
-    const GT* gs = reinterpret_cast<const GT*>(stage);
-    const float* es = reinterpret_cast<const float*>(stage + kGBytes);
-    const int local = warp * kSWarpElems + lane * 4;
     const uint64_t first = stream_element_index(t, warp, 0, lane, 0);
 #pragma unroll
     for (int v = 0; v < kSUnits; ++v) {
-      GradVec<GT> gv;
-      if constexpr (sizeof(GT) == 4)
-        gv.v = *reinterpret_cast<const float4*>(gs + local + v * 128);
-      else
-        gv.v = *reinterpret_cast<const uint2*>(gs + local + v * 128);
-      const float4 ev = *reinterpret_cast<const float4*>(es + local + v * 128);
-      a[v][0] = __fmaf_rn(gamma, gv[0], ev.x);
-      a[v][1] = __fmaf_rn(gamma, gv[1], ev.y);
-      a[v][2] = __fmaf_rn(gamma, gv[2], ev.z);
-      a[v][3] = __fmaf_rn(gamma, gv[3], ev.w);
-      st_stream_f4(e + first + v * 128, make_float4(a[v][0], a[v][1], a[v][2], a[v][3]));
+      this->accumulate(stage, warp * kSWarpElems + lane * 4 + v * 128, gamma, a[v]);
+      st_stream_f4(this->e + first + v * 128, make_float4(a[v][0], a[v][1], a[v][2], a[v][3]));
     }
     select(t, first, a, sel);
   }
@@ -308,34 +292,22 @@ struct LwCandOp {
       for (int j = 0; j < 4; ++j) {
         const uint64_t i = first + v * 128 + j;
         a[v][j] = 0.0f;
-        if (i < d) {
-          const float x = __fmaf_rn(gamma, grad_scalar(g, i), e[i]);
-          e[i] = x;
+        if (this->valid(i)) {
+          const float x = this->accumulate_at(i, gamma);
+          this->e[i] = x;
           a[v][j] = x;
         }
       }
     }
     select(t, first, a, sel);
-    // lanes past d select nothing (their a is 0 but their segment is unknown)
+    // positions that are no coordinates select nothing (their segment is unknown)
 #pragma unroll
     for (int v = 0; v < kSUnits; ++v)
 #pragma unroll
       for (int j = 0; j < 4; ++j)
-        if (first + v * 128 + j >= d) sel[v] &= ~(0x11u << j);
+        if (!this->valid(first + v * 128 + j)) sel[v] &= ~(0x11u << j);
   }
 };
-
-// Inputs the bulk copies cannot take (not 16-byte aligned): a = fmaf(γ,g,e)
-// written over e with plain loads; every segment is then selected from e.
-template <typename GT>
-__global__ void __launch_bounds__(kThreads)
-    lw_accumulate_plain_kernel(const GT* __restrict__ g, float* __restrict__ e, float gamma,
-                               uint32_t d, uint32_t* other_state) {
-  clear_state(other_state);
-  for (uint64_t i = static_cast<uint64_t>(blockIdx.x) * kThreads + threadIdx.x; i < d;
-       i += static_cast<uint64_t>(gridDim.x) * kThreads)
-    e[i] = __fmaf_rn(gamma, grad_scalar(g, i), e[i]);
-}
 
 // ------------------------------------------------------------- 3 select
 struct LwArgs {
@@ -345,13 +317,14 @@ struct LwArgs {
   const uint32_t* work_seg;   // segment ids of the single CTAs, grouped by CTA
   LwTeamState* teams;
   const uint32_t* tile_base;  // [tiles + 1] list position of each tile's first candidate
+  uint32_t shift;             // tiles are cut from positions: coordinates plus shift
   const uint32_t* list_idx;   // ordered candidates of the streaming pass
   const float* list_val;
   const uint32_t* list_flags; // that pass's latched bits
   uint32_t* error;
   uint32_t* count_out;
   uint64_t wait_limit_ns;
-  uint32_t tiles, cap, use_list;
+  uint32_t tiles, cap;
   uint32_t total_k;
   double* err_out;            // optional ||e'||^2 of the step
   const double* stream_err;   // the streaming pass's share (final residuals)
@@ -371,14 +344,17 @@ struct Source {
 };
 __device__ Source segment_source(const LwArgs& a, const LwSeg& s, uint32_t si) {
   Source src{false, 0, s.hi - s.lo};
-  if (!a.use_list || __ldcg(a.mbound + si) >= kLwDeferred) return src;
-  const uint32_t tl = s.lo / kTileElems, th = s.hi / kTileElems;  // tl < tiles, th <= tiles
+  if (__ldcg(a.mbound + si) >= kLwDeferred) return src;
+  const uint64_t p_lo = static_cast<uint64_t>(s.lo) + a.shift;
+  const uint64_t p_hi = static_cast<uint64_t>(s.hi) + a.shift;
+  const uint32_t tl = static_cast<uint32_t>(p_lo / kTileElems);  // < tiles
+  const uint32_t th = static_cast<uint32_t>(p_hi / kTileElems);  // <= tiles
   const uint32_t p0 = __ldcg(a.tile_base + tl), p1 = __ldcg(a.tile_base + tl + 1);
   const uint32_t q0 = __ldcg(a.tile_base + th);
   const uint32_t q1 = th < a.tiles ? __ldcg(a.tile_base + th + 1) : q0;
   // candidates of the partial tiles that lie below lo / hi (none to scan
   // when lo / hi starts a tile); a tile cut off at the capacity disqualifies
-  const uint32_t e0 = s.lo % kTileElems ? p1 : p0, e1 = s.hi % kTileElems ? q1 : q0;
+  const uint32_t e0 = p_lo % kTileElems ? p1 : p0, e1 = p_hi % kTileElems ? q1 : q0;
   if (e0 > a.cap || e1 > a.cap) return src;
   const uint32_t n0 = e0 - p0, n1 = e1 - q0, span = n0 > n1 ? n0 : n1;
   uint32_t below0 = 0, below1 = 0;
@@ -811,10 +787,10 @@ __global__ void __launch_bounds__(kLwThreads, 1)
 }
 
 // ------------------------------------------------------------- host side
-template <typename GT>
+template <typename GT, bool kAny>
 int lw_group_blocks_per_sm() {
-  const void* fn = reinterpret_cast<const void*>(&lookback_stream_kernel<LwCandOp<GT>, kLwStages>);
-  const uint32_t smem = LbLayout<LwCandOp<GT>, kLwStages>::kSmem;
+  const void* fn = reinterpret_cast<const void*>(&lookback_stream_kernel<LwCandOp<GT, kAny>, kLwStages>);
+  const uint32_t smem = LbLayout<LwCandOp<GT, kAny>, kLwStages>::kSmem;
   int n = 0;
   if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fn, kLbThreads, smem) != cudaSuccess)
@@ -823,10 +799,10 @@ int lw_group_blocks_per_sm() {
   return n;
 }
 
-template <typename GT>
+template <typename GT, bool kAny>
 int lw_stream_blocks_per_sm() {
-  const void* fn = reinterpret_cast<const void*>(&stream_compact_kernel<LwCandOp<GT>, kLwStages>);
-  const uint32_t smem = StreamLayout<LwCandOp<GT>, kLwStages>::kSmem;
+  const void* fn = reinterpret_cast<const void*>(&stream_compact_kernel<LwCandOp<GT, kAny>, kLwStages>);
+  const uint32_t smem = StreamLayout<LwCandOp<GT, kAny>, kLwStages>::kSmem;
   int n = 0;
   if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fn, kStreamThreads, smem) != cudaSuccess)
@@ -845,7 +821,7 @@ uint64_t select_cost(const LwSeg& s) {
   return 3ull * s.k + 4096;  // sampled: about 1.5 k_s candidates, a few passes
 }
 
-template <typename GT>
+template <bool kAny, typename GT>
 cudaError_t launch_typed(const GT* g, float* e, float gamma, uint32_t d, uint32_t* idx_out,
                          float* val_out, uint32_t* count_out, double* err_out, Workspace& ws,
                          const DeviceInfo& dev) {
@@ -863,67 +839,58 @@ cudaError_t launch_typed(const GT* g, float* e, float gamma, uint32_t d, uint32_
   uint32_t* tile_base = reinterpret_cast<uint32_t*>(p.dev + p.off_tile_base);
 
   const int per_sm = sizeof(GT) == 4 ? dev.lw_stream_per_sm_f32 : dev.lw_stream_per_sm_bf16;
-  const bool streamable = reinterpret_cast<uintptr_t>(e) % 16 == 0 &&
-                          reinterpret_cast<uintptr_t>(g) % 16 == 0 && per_sm > 0;
-  if (streamable) {
-    // 1 sample
-    if (p.n_sampled > 0) {
-      const uint2* sampled = reinterpret_cast<const uint2*>(p.dev + p.off_samples);
-      uint32_t cap = ws.cand_cap;
-      // the merged histograms of the multi-part segments: two copies, by call parity
-      uint32_t* part_hist = reinterpret_cast<uint32_t*>(p.dev + p.off_part_hist) +
-                            static_cast<size_t>(lw_parity & 1u) * p.n_part_hist * kLwPartHistWords;
-      void* sp[] = {(void*)&g, (void*)&e, (void*)&gamma, (void*)&segs, (void*)&sampled,
-                    (void*)&mbound, (void*)&cap, (void*)&part_hist};
-      err = launch_pdl(reinterpret_cast<const void*>(&lw_sample_kernel<GT>), p.n_sampled,
-                       kSampleThreads, kLwSampleSmem, ws.stream, sp, false);
-      count_launch();
-      if (err != cudaSuccess) return err;
-    }
-    // 2 stream
-    ScanCtx ctx = next_scan_ctx(ws, p.tiles);
-    ctx.error = list_flags;
-    LwCandOp<GT> op{g, e, gamma, d,
-                    reinterpret_cast<const uint32_t*>(p.dev + p.off_seg_end), mbound,
-                    reinterpret_cast<const uint32_t*>(p.dev + p.off_tile_info), other};
-    uint32_t slots = static_cast<uint32_t>(per_sm * dev.sm_count);
-    if (slots > kMaxChunks) slots = kMaxChunks;
-    const uint32_t grid = p.tiles < slots ? p.tiles : slots;
+  if (per_sm <= 0) return cudaErrorInvalidConfiguration;
+  StreamIn<GT, kAny> in = stream_in<GT, kAny>(g, e, d);
+  const uint32_t tiles = tiles_for(in.end);  // at most one more than the plan's
+  // 1 sample
+  if (p.n_sampled > 0) {
+    const uint2* sampled = reinterpret_cast<const uint2*>(p.dev + p.off_samples);
     uint32_t cap = ws.cand_cap;
-    uint32_t* list_count = ws.u32(kOffTkListCount);
-    const int per_sm_groups =
-        sizeof(GT) == 4 ? dev.lw_group_per_sm_f32 : dev.lw_group_per_sm_bf16;
-    if (use_group_kernel(p.tiles) && per_sm_groups > 0) {
-      // claimed groups of tiles with look-back (stream_lookback.cuh): no
-      // wait depends on which CTAs are resident
-      const uint32_t groups = (p.tiles + kLbGroupTiles - 1) / kLbGroupTiles;
-      const uint32_t gslots = static_cast<uint32_t>(per_sm_groups * dev.sm_count);
-      const uint32_t ggrid = groups < gslots ? groups : gslots;
-      LbArgs la{tile_base, err_out ? ws.stream_err() : nullptr, reinterpret_cast<FF*>(ws.counts()),
-                ws.stage_idx(), ws.stage_val()};
-      void* gp[] = {&op, &d, &list_idx, &list_val, &list_count, &cap, &ctx, &la};
-      err = launch_pdl(
-          reinterpret_cast<const void*>(&lookback_stream_kernel<LwCandOp<GT>, kLwStages>), ggrid,
-          kLbThreads, LbLayout<LwCandOp<GT>, kLwStages>::kSmem, ws.stream, gp, false);
-    } else {
-      StreamArgs sa{ws.stage_idx(), ws.stage_val(), ws.counts(), ws.chunks(), tile_base,
-                    err_out ? ws.stream_err() : nullptr, ws.errparts()};
-      void* params[] = {&op, &d, &list_idx, &list_val, &list_count, &cap, &ctx, &sa};
-      // not cooperative: the only cross-CTA wait is on lower-numbered CTAs,
-      // which are scheduled first
-      err = launch_pdl(
-          reinterpret_cast<const void*>(&stream_compact_kernel<LwCandOp<GT>, kLwStages>), grid,
-          kStreamThreads, StreamLayout<LwCandOp<GT>, kLwStages>::kSmem, ws.stream, params, false);
-    }
+    // the merged histograms of the multi-part segments: two copies, by call parity
+    uint32_t* part_hist = reinterpret_cast<uint32_t*>(p.dev + p.off_part_hist) +
+                          static_cast<size_t>(lw_parity & 1u) * p.n_part_hist * kLwPartHistWords;
+    void* sp[] = {(void*)&in, (void*)&gamma, (void*)&segs, (void*)&sampled,
+                  (void*)&mbound, (void*)&cap, (void*)&part_hist};
+    err = launch_pdl(reinterpret_cast<const void*>(&lw_sample_kernel<GT, kAny>), p.n_sampled,
+                     kSampleThreads, kLwSampleSmem, ws.stream, sp, false);
     count_launch();
     if (err != cudaSuccess) return err;
-  } else {
-    const uint32_t grid = p.tiles < static_cast<uint32_t>(dev.sm_count * 8)
-                              ? p.tiles : static_cast<uint32_t>(dev.sm_count * 8);
-    lw_accumulate_plain_kernel<GT><<<grid, kThreads, 0, ws.stream>>>(g, e, gamma, d, other);
-    count_launch();
-    if ((err = cudaGetLastError()) != cudaSuccess) return err;
   }
+  // 2 stream
+  ScanCtx ctx = next_scan_ctx(ws, tiles);
+  ctx.error = list_flags;
+  LwCandOp<GT, kAny> op{in, gamma, reinterpret_cast<const uint32_t*>(p.dev + p.off_seg_end), mbound,
+                  reinterpret_cast<const uint32_t*>(p.dev + p.off_tile_info), p.tiles, other};
+  uint32_t slots = static_cast<uint32_t>(per_sm * dev.sm_count);
+  if (slots > kMaxChunks) slots = kMaxChunks;
+  const uint32_t grid = tiles < slots ? tiles : slots;
+  uint32_t cap = ws.cand_cap;
+  uint32_t* list_count = ws.u32(kOffTkListCount);
+  const int per_sm_groups = sizeof(GT) == 4 ? dev.lw_group_per_sm_f32 : dev.lw_group_per_sm_bf16;
+  if (use_group_kernel(tiles) && per_sm_groups > 0) {
+    // claimed groups of tiles with look-back (stream_lookback.cuh): no
+    // wait depends on which CTAs are resident
+    const uint32_t groups = (tiles + kLbGroupTiles - 1) / kLbGroupTiles;
+    const uint32_t gslots = static_cast<uint32_t>(per_sm_groups * dev.sm_count);
+    const uint32_t ggrid = groups < gslots ? groups : gslots;
+    LbArgs la{tile_base, err_out ? ws.stream_err() : nullptr, reinterpret_cast<FF*>(ws.counts()),
+              ws.stage_idx(), ws.stage_val()};
+    void* gp[] = {&op, &list_idx, &list_val, &list_count, &cap, &ctx, &la};
+    err = launch_pdl(
+        reinterpret_cast<const void*>(&lookback_stream_kernel<LwCandOp<GT, kAny>, kLwStages>), ggrid,
+        kLbThreads, LbLayout<LwCandOp<GT, kAny>, kLwStages>::kSmem, ws.stream, gp, false);
+  } else {
+    StreamArgs sa{ws.stage_idx(), ws.stage_val(), ws.counts(), ws.chunks(), tile_base,
+                  err_out ? ws.stream_err() : nullptr, ws.errparts()};
+    void* cp[] = {&op, &list_idx, &list_val, &list_count, &cap, &ctx, &sa};
+    // not cooperative: the only cross-CTA wait is on lower-numbered CTAs,
+    // which are scheduled first
+    err = launch_pdl(
+        reinterpret_cast<const void*>(&stream_compact_kernel<LwCandOp<GT, kAny>, kLwStages>), grid,
+        kStreamThreads, StreamLayout<LwCandOp<GT, kAny>, kLwStages>::kSmem, ws.stream, cp, false);
+  }
+  count_launch();
+  if (err != cudaSuccess) return err;
   // 3 select: a cooperative launch when there are teams, so that every
   // team's CTAs are resident
   LwArgs a;
@@ -939,12 +906,11 @@ cudaError_t launch_typed(const GT* g, float* e, float gamma, uint32_t d, uint32_
   a.error = ws.u32(kOffError);
   a.count_out = count_out;
   a.wait_limit_ns = wait_limit_ns();
-  a.tiles = p.tiles;
+  a.shift = in.shift_;
+  a.tiles = tiles;
   a.cap = ws.cand_cap;
-  a.use_list = streamable ? 1u : 0u;
   a.total_k = static_cast<uint32_t>(p.total_k);
-  // inputs the streaming pass could not take: the norm by a plain pass after
-  a.err_out = streamable ? err_out : nullptr;
+  a.err_out = err_out;
   a.stream_err = ws.stream_err();
   a.err_parts = ws.errparts();
   a.err_arrive = state + kStErrArrive / 4;
@@ -953,7 +919,6 @@ cudaError_t launch_typed(const GT* g, float* e, float gamma, uint32_t d, uint32_
   err = launch_pdl(reinterpret_cast<const void*>(&lw_select_kernel), p.n_select_ctas, kLwThreads,
                    kLwSelectSmem, ws.stream, params, p.n_teams > 0);
   count_launch();
-  if (err == cudaSuccess && err_out && !streamable) err = launch_error_norm(e, d, err_out, ws, dev);
   return err;
 }
 
@@ -963,10 +928,12 @@ void topk_layerwise_init_device(DeviceInfo& info) {
   int n = 0;
   // the sampling kernel's histogram (dynamic shared memory); a failure here
   // makes its launches fail, which the calls report
-  cudaFuncSetAttribute(lw_sample_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       kLwSampleSmem);
-  cudaFuncSetAttribute(lw_sample_kernel<uint16_t>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       kLwSampleSmem);
+  const void* samplers[] = {reinterpret_cast<const void*>(&lw_sample_kernel<float, false>),
+                            reinterpret_cast<const void*>(&lw_sample_kernel<float, true>),
+                            reinterpret_cast<const void*>(&lw_sample_kernel<uint16_t, false>),
+                            reinterpret_cast<const void*>(&lw_sample_kernel<uint16_t, true>)};
+  for (const void* f : samplers)
+    cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kLwSampleSmem);
   cudaGetLastError();
   if (cudaFuncSetAttribute(lw_select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            kLwSelectSmem) != cudaSuccess ||
@@ -974,10 +941,14 @@ void topk_layerwise_init_device(DeviceInfo& info) {
                                                     kLwSelectSmem) != cudaSuccess)
     n = 0;
   info.lw_select_per_sm = n;
-  info.lw_stream_per_sm_f32 = lw_stream_blocks_per_sm<float>();
-  info.lw_stream_per_sm_bf16 = lw_stream_blocks_per_sm<uint16_t>();
-  info.lw_group_per_sm_f32 = lw_group_blocks_per_sm<float>();
-  info.lw_group_per_sm_bf16 = lw_group_blocks_per_sm<uint16_t>();
+  info.lw_stream_per_sm_f32 =
+      std::min(lw_stream_blocks_per_sm<float, false>(), lw_stream_blocks_per_sm<float, true>());
+  info.lw_stream_per_sm_bf16 =
+      std::min(lw_stream_blocks_per_sm<uint16_t, false>(), lw_stream_blocks_per_sm<uint16_t, true>());
+  info.lw_group_per_sm_f32 =
+      std::min(lw_group_blocks_per_sm<float, false>(), lw_group_blocks_per_sm<float, true>());
+  info.lw_group_per_sm_bf16 =
+      std::min(lw_group_blocks_per_sm<uint16_t, false>(), lw_group_blocks_per_sm<uint16_t, true>());
   cudaGetLastError();
 }
 
@@ -1164,7 +1135,7 @@ cudaError_t lw_prepare(Workspace& ws, const uint64_t* seg_end, const uint64_t* s
   p.off_teams = take(sizeof(LwTeamState) * n_teams);
   p.off_part_hist = take(2 * sizeof(uint32_t) * kLwPartHistWords * n_part_hist);
   const size_t zero_end = off;
-  p.off_tile_base = take(sizeof(uint32_t) * (tiles + 1));
+  p.off_tile_base = take(sizeof(uint32_t) * (tiles + 2));  // positions: perhaps a tile more
   p.total = off;
 
   p.image.assign(upload, 0);
@@ -1219,11 +1190,13 @@ cudaError_t lw_prepare(Workspace& ws, const uint64_t* seg_end, const uint64_t* s
 cudaError_t launch_topk_layerwise(const void* g, bool g_bf16, float* e, float gamma, uint32_t d,
                                   uint32_t* idx_out, float* val_out, uint32_t* count_out,
                                   double* err_out, Workspace& ws, const DeviceInfo& dev) {
-  if (g_bf16)
-    return launch_typed(static_cast<const uint16_t*>(g), e, gamma, d, idx_out, val_out,
-                        count_out, err_out, ws, dev);
-  return launch_typed(static_cast<const float*>(g), e, gamma, d, idx_out, val_out, count_out,
-                      err_out, ws, dev);
+  auto run = [&](auto* gt) {
+    return positions(gt, e).any() ? launch_typed<true>(gt, e, gamma, d, idx_out, val_out,
+                                                       count_out, err_out, ws, dev)
+                                  : launch_typed<false>(gt, e, gamma, d, idx_out, val_out,
+                                                        count_out, err_out, ws, dev);
+  };
+  return g_bf16 ? run(static_cast<const uint16_t*>(g)) : run(static_cast<const float*>(g));
 }
 
 }  // namespace efs
