@@ -9,9 +9,11 @@
 // every coordinate receives its contributions in ascending worker order —
 // the same fp32 sum as the plain sequential loop.
 //
-// Kernel 1 finds, by binary search, where each worker's sorted list crosses
-// each tile boundary; kernel 2 does the reduction and writes each dense tile
-// once with 16-byte stores. Traffic: 8 B per pair read + 4 B per coordinate
+// Kernel 1 finds where each worker's sorted list crosses each tile boundary
+// (not needed when the messages come with their tile indexes); kernel 2 does
+// the reduction and writes each dense tile once with 16-byte stores: a CTA per
+// tile as above, or for a plain sum of up to 32 workers over many tiles one
+// warp per tile (agg_stream_kernel), where worker order needs no barriers. Traffic: 8 B per pair read + 4 B per coordinate
 // written (+ the small offsets table).
 //
 // The same reduction can instead end in the model update that follows the
@@ -21,7 +23,11 @@
 // gradient compression). The dense sum then never reaches memory: 8 B per
 // coordinate (read and write x), 16 B with momentum, instead of writing the
 // sum and a second pass that reads it back.
+#include <algorithm>
+#include <cstddef>
+
 #include "internal.h"
+#include "tma.cuh"
 
 namespace efs {
 namespace {
@@ -34,17 +40,24 @@ struct AggPtrs {
 
 // off[i * (tiles + 1) + t] = number of entries of list i below t * kAggTile;
 // off[i * (tiles + 1) + tiles] = counts[i]. Grid: blockIdx.y = list, x over
-// the tiles + 1 entries. Two ways to the same numbers, chosen per list:
-//  - a list with at least (tiles + 1) / 16 and at most 8 (tiles + 1) entries
-//    is scattered: entry p (p = 0..count, count standing for the end) owns the
-//    tiles t with list[p - 1] < t * kAggTile <= list[p] and writes p there —
-//    two loads per entry and no dependent chain; a run of more than 8 tiles
-//    is written by the whole warp;
-//  - other lists: one binary search per tile (14-23 dependent loads, but
-//    independent of the list's length).
+// the tiles + 1 entries. Two ways to the same numbers:
+//  - scattered, when the lists hold at most kScatterEntries entries together
+//    and this one at least (tiles + 1) / 16: entry p (p = 0..count, count
+//    standing for the end) owns the tiles t with
+//    list[p - 1] < t * kAggTile <= list[p] and writes p there. A thread reads
+//    4 consecutive entries and the one before them, nothing waits for
+//    anything else; a run of more than 8 tiles is written by the whole warp;
+//  - otherwise one binary search per tile (14-23 dependent loads, but
+//    independent of the lists' length).
 // Either way every entry lies in [0, count]; a list that is not strictly
 // ascending is latched as bad input (scatter) and may leave entries the
 // reduction clamps to the list.
+// The scatter reads every index once (32 MB at most, about 8 us), the searches
+// take 8 to 12 us whatever the lists hold. Measured, us an exchange, searches
+// -> scatter: 16 lists of 256 K entries over 6,240 tiles 61.6 -> 54.8, 4
+// LSTM-shaped workers' steps with their exchange (0.9 M entries each) 333.5 ->
+// 300.2.
+constexpr uint32_t kScatterEntries = 8u << 20;
 __global__ void __launch_bounds__(kThreads)
     agg_offsets_kernel(AggPtrs p, const uint32_t* __restrict__ counts, uint32_t n,
                        uint32_t tiles, uint32_t* __restrict__ off, uint32_t* __restrict__ error) {
@@ -55,11 +68,13 @@ __global__ void __launch_bounds__(kThreads)
   const uint32_t tx = blockIdx.x * kThreads + threadIdx.x;
   const uint32_t stride = gridDim.x * kThreads;  // >= per
   const int lane = threadIdx.x & 31;
+  uint32_t all = 0;  // entries of all lists (each clamped: 256 of them fit)
+  for (uint32_t q = lane; q < n; q += 32) all += min(counts[q], 1u << 23);
+  all = warp_sum(all);
   const uint32_t cnt = counts[i];
   const uint32_t* x = p.idx[i];
   uint32_t* o = off + static_cast<uint64_t>(i) * per;
-  const bool scatter = cnt >= per / 16 && static_cast<uint64_t>(cnt) <= 8ull * per;
-  if (!scatter) {
+  if (cnt < per / 16 || all > kScatterEntries) {
     if (tx >= per) return;
     uint32_t result = cnt;
     if (tx < tiles) {
@@ -78,31 +93,47 @@ __global__ void __launch_bounds__(kThreads)
     return;
   }
   bool bad = false;
+  const bool vec = (reinterpret_cast<uintptr_t>(x) & 15u) == 0;
+  const uint32_t quads = cnt / 4 + 1;  // positions 0..cnt
 #pragma unroll 1
-  for (uint32_t q = 0; q < 9; ++q) {  // positions tx + q * stride <= cnt (cnt <= 8 per)
-    const uint32_t pos = tx + q * stride;
-    const bool has = pos <= cnt;
-    uint32_t t_lo = 1, t_hi = 0;  // empty
-    if (has) {
-      const uint32_t cur = pos < cnt ? __ldg(x + pos) : 0u;
-      const uint32_t prev = pos > 0 ? __ldg(x + pos - 1) : 0u;
-      if (pos > 0 && pos < cnt && prev >= cur) bad = true;  // not strictly ascending
-      t_lo = pos == 0 ? 0u : min(prev / kAggTile + 1u, per);
-      t_hi = pos == cnt ? tiles : min(cur / kAggTile, tiles - 1u);
-      if (pos < cnt && t_hi < t_lo) t_lo = t_hi + 1;  // nothing (malformed, or a shared tile)
+  for (uint32_t g0 = blockIdx.x * kThreads + (threadIdx.x & ~31u); g0 < quads; g0 += stride) {
+    const uint32_t p0 = (g0 + lane) * 4;
+    uint32_t v[5];  // the entry before p0, then entries p0 .. p0 + 3
+    v[0] = p0 > 0 && p0 <= cnt ? __ldg(x + p0 - 1) : 0u;
+    if (vec && p0 + 4 <= cnt) {
+      const uint4 w = __ldg(reinterpret_cast<const uint4*>(x + p0));
+      v[1] = w.x, v[2] = w.y, v[3] = w.z, v[4] = w.w;
+    } else {
+#pragma unroll
+      for (int u = 0; u < 4; ++u) v[1 + u] = p0 + u < cnt ? __ldg(x + p0 + u) : 0u;
     }
-    const bool mine = has && t_lo <= t_hi && t_hi - t_lo < 8;
-    if (mine)
-      for (uint32_t t = t_lo; t <= t_hi; ++t) o[t] = pos;
-    // longer runs: the whole warp writes them, one run after another
-    uint32_t m = __ballot_sync(0xffffffffu, has && t_lo <= t_hi && !mine);
-    while (m) {
-      const int l = __ffs(m) - 1;
-      m &= m - 1;
-      const uint32_t a = __shfl_sync(0xffffffffu, t_lo, l);
-      const uint32_t b = __shfl_sync(0xffffffffu, t_hi, l);
-      const uint32_t v = __shfl_sync(0xffffffffu, pos, l);
-      for (uint32_t t = a + lane; t <= b; t += 32) o[t] = v;
+    bool far = false;
+    uint32_t t_lo[4], t_hi[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const uint32_t pos = p0 + u;
+      t_lo[u] = pos == 0 ? 0u : min(v[u] / kAggTile + 1u, per);
+      t_hi[u] = pos == cnt ? tiles : min(v[u + 1] / kAggTile, tiles - 1u);
+      if (pos > cnt) t_lo[u] = t_hi[u] + 1;  // nothing
+      if (pos > 0 && pos < cnt && v[u] >= v[u + 1]) bad = true;  // not strictly ascending
+      if (t_lo[u] > t_hi[u]) continue;  // a shared tile (or malformed): nothing
+      if (t_hi[u] - t_lo[u] < 8)
+        for (uint32_t t = t_lo[u]; t <= t_hi[u]; ++t) o[t] = pos;
+      else
+        far = true;
+    }
+    if (!__any_sync(0xffffffffu, far)) continue;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {  // longer runs: the whole warp writes them, one after another
+      uint32_t m = __ballot_sync(0xffffffffu, t_lo[u] <= t_hi[u] && t_hi[u] - t_lo[u] >= 8);
+      while (m) {
+        const int l = __ffs(m) - 1;
+        m &= m - 1;
+        const uint32_t a = __shfl_sync(0xffffffffu, t_lo[u], l);
+        const uint32_t b = __shfl_sync(0xffffffffu, t_hi[u], l);
+        const uint32_t pos = __shfl_sync(0xffffffffu, p0 + u, l);
+        for (uint32_t t = a + lane; t <= b; t += 32) o[t] = pos;
+      }
     }
   }
   if (bad) atomicOr(error, kDevErrBadInput);
@@ -266,6 +297,259 @@ __global__ void __launch_bounds__(kThreads)
   }
 }
 
+// ---------------------------------------------- the dense sum, many tiles
+// One warp per CTA, persistent, a tile at a time: the warp keeps the tile's
+// sum in shared memory and adds worker 0's pairs, then worker 1's, ... — a
+// single warp needs no barrier between workers —, while the next pairs are on
+// their way. Lane i holds worker i's list: it fetches the offsets of its next
+// run a tile ahead and copies the run's aligned 16-byte windows of indices
+// and values with one bulk copy each into a stage of kAggPairs pairs (a tile
+// whose runs need more takes several stages; the windows are laid out in
+// worker order). A lane then takes 4 consecutive pairs at a time (two
+// 16-byte reads), so that 128 pairs cost about 45 instructions.
+//
+// Why: with a CTA of 8 warps per tile (agg_reduce_kernel) the reduction was
+// bound by instructions, not by memory: 8,200 warp instructions a tile of
+// 1,640 pairs (issue slots 77 % busy, DRAM at 27 %), most of them the loops
+// and barriers around a few pairs per warp and worker. Here the same tile
+// takes about 1,500, and what bounds it is the latency of the shared-memory
+// reads of 8 warps an SM (16 KB of sums each), or DRAM once tiles hold many
+// pairs. Measured on a GB300, us an exchange, before -> after: 8 workers'
+// hard-threshold messages at 5 % of d = 138.4 M, with tile indexes, 262 ->
+// 164 (6.1 TB/s, 91 % of the copy rate); 16 workers' Top-k messages at 1 % of
+// d = 25.6 M, 51.8 -> 49.2. Stages of 448, 544, 768, 896 and 1,792 pairs:
+// 175, 171, 183, 169 and 192 on the first, 61, 52, 62, 56 and 55 on the
+// second. Copies by cp.async instead of bulk copies (more instructions of the
+// one warp): 194-236 and 62-66.
+constexpr uint32_t kAggPairs = 640;   // pairs a stage holds
+constexpr int kAggStages = 2;          // one being added, one on its way
+// From this many tiles on (6 per SM): with fewer, warps would be left without
+// a tile while others take two, and a CTA of 8 warps finishes a tile sooner.
+constexpr uint32_t kAggMinTiles = 912;
+
+struct AggStream {  // shared memory of a CTA
+  float acc[kAggTile + 32];  // the tile's sum; one unused slot per lane
+  uint32_t idx[kAggStages][kAggPairs];
+  float val[kAggStages][kAggPairs];
+  uint32_t run[kAggStages][32];  // worker's first pair in the stage | pairs << 16
+  uint32_t tile[kAggStages], last[kAggStages];
+  uint64_t bar[kAggStages];
+};
+static_assert(offsetof(AggStream, idx) % 16 == 0 && offsetof(AggStream, val) % 16 == 0 &&
+                  offsetof(AggStream, bar) % 8 == 0 && kAggPairs % 4 == 0,
+              "bulk copies");
+
+template <bool kVec>
+__global__ void __launch_bounds__(32)
+    agg_stream_kernel(AggPtrs p, uint32_t n, uint32_t d, uint32_t tiles,
+                      const uint32_t* __restrict__ off, const uint32_t* __restrict__ counts,
+                      float* __restrict__ out, uint32_t* __restrict__ error,
+                      uint64_t wait_limit_ns) {
+  extern __shared__ __align__(128) unsigned char smem[];
+  AggStream& sm = *reinterpret_cast<AggStream*>(smem);
+  const uint32_t lane = threadIdx.x;
+  if (lane == 0) {
+    for (int s = 0; s < kAggStages; ++s) mbar_init(&sm.bar[s], 1);
+    mbar_init_fence();
+  }
+  for (uint32_t q = lane; q < kAggTile / 4; q += 32)
+    reinterpret_cast<float4*>(sm.acc)[q] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+  __syncwarp();
+  griddep_wait();  // the lists and offsets (and everything before them) are complete
+  griddep_launch_dependents();
+  const bool has = lane < n;
+  const uint32_t* const li = has ? p.idx[lane] : nullptr;
+  const float* const lv = has ? p.val[lane] : nullptr;
+  const uint32_t* const r =
+      !has ? nullptr : off ? off + static_cast<uint64_t>(lane) * (tiles + 1) : p.tiles[lane];
+  const uint32_t count = has ? counts[lane] : 0u;
+  const bool bulk =
+      ((reinterpret_cast<uintptr_t>(li) | reinterpret_cast<uintptr_t>(lv)) & 15u) == 0;
+  const uint64_t policy = l2_evict_normal_policy();
+  bool bad = false;
+
+  // the tile whose pairs are copied next: this lane's run [lo, lo + cnt), its
+  // place `base` in the tile's sequence of windows, and the sequence's
+  // length; and the offsets read for the tile after it
+  uint32_t next = blockIdx.x, lo = 0, cnt = 0, base = 0, total = 0, b0 = 0;
+  uint32_t r0 = 0, r1 = 0;
+  auto fetch = [&](uint32_t t) {
+    if (has && t < tiles) {
+      r0 = __ldg(r + t);
+      r1 = __ldg(r + t + 1);
+    }
+  };
+  auto enter = [&]() {  // tile `next`, whose offsets were fetched
+    lo = min(r0, count);
+    const uint32_t hi = min(r1, count);  // never past the list
+    cnt = hi > lo ? hi - lo : 0u;
+    if (cnt > kAggTile) {  // more than a tile can hold: not a tile's run
+      cnt = kAggTile;
+      bad = true;
+    }
+    const uint32_t len = cnt ? ((lo & 3u) + cnt + 3u) & ~3u : 0u;
+    uint32_t incl = len;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t x = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= static_cast<uint32_t>(o)) incl += x;
+    }
+    base = incl - len;
+    total = __shfl_sync(0xffffffffu, incl, 31);
+    b0 = 0;
+    fetch(next + gridDim.x);
+  };
+  fetch(next);
+  if (next < tiles) enter();
+
+  // copies the next pairs into stage s; false when there are no more tiles
+  auto issue = [&](uint32_t s) -> bool {
+    if (next >= tiles) return false;
+    const uint32_t head = base + (lo & 3u);
+    const uint32_t y0 = max(head, b0), y1 = min(head + cnt, b0 + kAggPairs);
+    const bool some = y1 > y0;
+    const uint32_t x0 = (y0 & ~3u) - b0, x1 = ((y1 + 3u) & ~3u) - b0;  // in the stage
+    sm.run[s][lane] = some ? (y0 - b0) | ((y1 - y0) << 16) : 0u;
+    const uint32_t src = (lo & ~3u) + (b0 + x0 - base);  // list position of x0
+    const uint32_t bytes = some && bulk ? (x1 - x0) * 4u : 0u;
+    const uint32_t tx = 2u * warp_sum(bytes);
+    if (lane == 0) {
+      sm.tile[s] = next;
+      sm.last[s] = b0 + kAggPairs >= total ? 1u : 0u;
+      mbar_arrive_expect_tx(&sm.bar[s], tx);
+    }
+    __syncwarp();
+    if (bytes) {
+      tma_load_1d(&sm.idx[s][x0], li + src, bytes, &sm.bar[s], policy);
+      tma_load_1d(&sm.val[s][x0], lv + src, bytes, &sm.bar[s], policy);
+    }
+    uint32_t plain = __ballot_sync(0xffffffffu, some && !bulk);
+    if (plain) {  // lists that are not 16-byte aligned: by plain loads
+      while (plain) {
+        const int q = __ffs(plain) - 1;
+        plain &= plain - 1;
+        const uint32_t run = sm.run[s][q];
+        const uint32_t a = run & 0xffffu, z = a + (run >> 16);
+        const uint32_t at = __shfl_sync(0xffffffffu, src + (y0 & 3u), q);
+        const uint32_t* qi = p.idx[q];
+        const float* qv = p.val[q];
+        for (uint32_t x = a + lane; x < z; x += 32) {
+          sm.idx[s][x] = __ldg(qi + at + (x - a));
+          sm.val[s][x] = __ldg(qv + at + (x - a));
+        }
+      }
+      // these writes before the stage's next bulk copies
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      __syncwarp();
+    }
+    if (b0 + kAggPairs >= total) {
+      next += gridDim.x;
+      if (next < tiles) enter();
+    } else {
+      b0 += kAggPairs;
+    }
+    return true;
+  };
+
+  bool more = true;
+  uint32_t issued = 0, done = 0;
+  while (true) {
+    while (more && issued - done < static_cast<uint32_t>(kAggStages)) {
+      more = issue(issued % kAggStages);
+      if (more) ++issued;
+    }
+    if (done == issued) break;
+    const uint32_t s = done % kAggStages;
+    if (!__all_sync(0xffffffffu, mbar_wait(&sm.bar[s], (done / kAggStages) & 1u, wait_limit_ns))) {
+      if (lane == 0) atomicOr(error, kDevErrTimeout);
+      break;
+    }
+    const uint32_t tile = sm.tile[s];
+    const uint64_t j0 = static_cast<uint64_t>(tile) * kAggTile;
+    const uint32_t room = static_cast<uint32_t>(min(d - j0, static_cast<uint64_t>(kAggTile)));
+    const uint32_t my_run = sm.run[s][lane];
+    uint32_t live = __ballot_sync(0xffffffffu, my_run >> 16);
+    // the stage's pairs, 128 at a time, worker by worker: (first, end) of the
+    // worker's run and this lane's 4 pairs from x on, read one step ahead
+    struct Quad {
+      uint4 j;
+      float4 v;
+      uint32_t x, first, len;
+    };
+    uint32_t q_first = 0, q_end = 0, q_x = 0;
+    auto read = [&](Quad& c) -> bool {
+      if (q_x >= q_end) {
+        if (!live) return false;
+        const uint32_t run = __shfl_sync(0xffffffffu, my_run, __ffs(live) - 1);
+        live &= live - 1;
+        q_first = run & 0xffffu;
+        q_end = q_first + (run >> 16);
+        q_x = q_first & ~3u;
+      }
+      c.x = q_x + 4 * lane;
+      c.first = q_first;
+      c.len = q_end - q_first;
+      if (c.x < q_end) {
+        c.j = *reinterpret_cast<const uint4*>(&sm.idx[s][c.x]);
+        c.v = *reinterpret_cast<const float4*>(&sm.val[s][c.x]);
+      }
+      q_x += 128;
+      return true;
+    };
+    auto add = [&](const Quad& c) {
+      const uint32_t j[4] = {c.j.x, c.j.y, c.j.z, c.j.w};
+      const float v[4] = {c.v.x, c.v.y, c.v.z, c.v.w};
+      uint32_t at[4];
+      float sum[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const bool in_run = c.x + u - c.first < c.len;  // wraps before the run
+        const uint32_t rel = j[u] - static_cast<uint32_t>(j0);
+        // unsorted or out-of-range input: skipped, latched
+        const bool ok = in_run && rel < room;
+        bad |= in_run != ok;
+        at[u] = ok ? rel : kAggTile + lane;
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) sum[u] = sm.acc[at[u]];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) sm.acc[at[u]] = sum[u] + v[u];
+      __syncwarp();
+    };
+    Quad a, b;
+    bool have = read(a);
+    while (have) {
+      const bool have_b = read(b);
+      add(a);
+      if (!have_b) break;
+      have = read(a);
+      add(b);
+    }
+    if (sm.last[s]) {  // the tile is complete: write it, and zero the sum again
+      float4* acc4 = reinterpret_cast<float4*>(sm.acc);
+      if (kVec && room == kAggTile) {
+        float4* o4 = reinterpret_cast<float4*>(out + j0);
+#pragma unroll 8
+        for (uint32_t q = lane; q < kAggTile / 4; q += 32) {
+          o4[q] = acc4[q];
+          acc4[q] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        }
+      } else {
+        for (uint32_t q = lane; q < kAggTile; q += 32) {
+          if (q < room) out[j0 + q] = sm.acc[q];
+          sm.acc[q] = 0.0f;
+        }
+      }
+    }
+    __syncwarp();
+    ++done;
+  }
+  // no copy may land after the CTA exits (only after a wait ran out)
+  for (; done < issued; ++done)
+    mbar_wait(&sm.bar[done % kAggStages], (done / kAggStages) & 1u, wait_limit_ns);
+  if (bad) atomicOr(error, kDevErrBadInput);
+}
+
 template <int kMode>
 cudaError_t launch_reduce(bool vec, AggPtrs p, uint32_t n, uint32_t d, uint32_t tiles,
                           const uint32_t* off, const uint32_t* counts, AggOut o, Workspace& ws) {
@@ -278,7 +562,7 @@ cudaError_t launch_reduce(bool vec, AggPtrs p, uint32_t n, uint32_t d, uint32_t 
 
 cudaError_t launch_common(uint32_t n, const uint32_t* const* idx, const float* const* val,
                           const uint32_t* const* tile_index, const uint32_t* counts, uint32_t d,
-                          const AggOut& o, int mode, Workspace& ws) {
+                          const AggOut& o, int mode, Workspace& ws, int agg_stream_slots) {
   AggPtrs p;
   for (uint32_t i = 0; i < kMaxWorkers; ++i) {
     p.idx[i] = i < n ? idx[i] : nullptr;
@@ -289,7 +573,11 @@ cudaError_t launch_common(uint32_t n, const uint32_t* const* idx, const float* c
   cudaError_t err = cudaSuccess;
   uint32_t* off = nullptr;
   if (!tile_index) {  // locate each list's tile boundaries first
-    const dim3 grid1((tiles + 1 + kThreads - 1) / kThreads, n);
+    // a thread per tile for the searches; for the scatter about 8 CTAs per SM
+    // in all, but no more than 16 entries a tile would occupy
+    const uint32_t per_tile = (tiles + 1 + kThreads - 1) / kThreads;
+    const uint32_t wide = std::min((1216 + n - 1) / n, (tiles / kThreads + 1) * 16);
+    const dim3 grid1(std::max(per_tile, wide), n);
     off = ws.offsets();
     const uint32_t* counts_arg = counts;
     uint32_t n_arg = n, tiles_arg = tiles;
@@ -302,7 +590,19 @@ cudaError_t launch_common(uint32_t n, const uint32_t* const* idx, const float* c
   }
   const bool vec = reinterpret_cast<uintptr_t>(o.out) % 16 == 0 &&
                    reinterpret_cast<uintptr_t>(o.m) % 16 == 0;
-  if (mode == kAggDense)
+  if (mode == kAggDense && n <= 32 && tiles >= kAggMinTiles && agg_stream_slots > 0) {
+    uint32_t n_arg = n, tiles_arg = tiles;
+    const uint32_t* counts_arg = counts;
+    float* out = o.out;
+    uint32_t* error = ws.u32(kOffError);
+    uint64_t limit = wait_limit_ns();
+    void* params[] = {&p, &n_arg, &d, &tiles_arg, &off, &counts_arg, &out, &error, &limit};
+    const void* fn = vec ? reinterpret_cast<const void*>(&agg_stream_kernel<true>)
+                         : reinterpret_cast<const void*>(&agg_stream_kernel<false>);
+    const uint32_t slots = static_cast<uint32_t>(agg_stream_slots);
+    err = launch_pdl(fn, tiles < slots ? tiles : slots, 32, sizeof(AggStream), ws.stream, params,
+                     false);
+  } else if (mode == kAggDense)
     err = launch_reduce<kAggDense>(vec, p, n, d, tiles, off, counts, o, ws);
   else if (mode == kAggSgd)
     err = launch_reduce<kAggSgd>(vec, p, n, d, tiles, off, counts, o, ws);
@@ -313,7 +613,21 @@ cudaError_t launch_common(uint32_t n, const uint32_t* const* idx, const float* c
 }
 }  // namespace
 
-void aggregate_init_device() {
+void aggregate_init_device(DeviceInfo& info) {
+  const void* streams[] = {reinterpret_cast<const void*>(&agg_stream_kernel<true>),
+                           reinterpret_cast<const void*>(&agg_stream_kernel<false>)};
+  int per_sm = 0;
+  for (const void* f : streams) {
+    int b = 0;
+    cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout,
+                         cudaSharedmemCarveoutMaxShared);
+    if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, sizeof(AggStream)) !=
+            cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, f, 32, sizeof(AggStream)) != cudaSuccess)
+      b = 0;
+    per_sm = f == streams[0] || b < per_sm ? b : per_sm;
+  }
+  info.agg_stream_slots = per_sm * info.sm_count;
   const void* fns[] = {
       reinterpret_cast<const void*>(&agg_reduce_kernel<true, kAggDense>),
       reinterpret_cast<const void*>(&agg_reduce_kernel<false, kAggDense>),
@@ -329,9 +643,10 @@ void aggregate_init_device() {
 
 cudaError_t launch_aggregate(uint32_t n, const uint32_t* const* idx, const float* const* val,
                              const uint32_t* const* tiles, const uint32_t* counts, uint32_t d,
-                             float* dense_out, Workspace& ws) {
+                             float* dense_out, Workspace& ws, const DeviceInfo& dev) {
   return launch_common(n, idx, val, tiles, counts, d,
-                       AggOut{dense_out, nullptr, 1.0f, 0.0f, 0.0f}, kAggDense, ws);
+                       AggOut{dense_out, nullptr, 1.0f, 0.0f, 0.0f}, kAggDense, ws,
+                       dev.agg_stream_slots);
 }
 
 cudaError_t launch_aggregate_apply(uint32_t n, const uint32_t* const* idx,
@@ -339,7 +654,7 @@ cudaError_t launch_aggregate_apply(uint32_t n, const uint32_t* const* idx,
                                    const uint32_t* counts, uint32_t d, float alpha, float* x,
                                    float* m, float mu, float lr, Workspace& ws) {
   return launch_common(n, idx, val, tiles, counts, d, AggOut{x, m, alpha, mu, lr},
-                       m ? kAggMomentum : kAggSgd, ws);
+                       m ? kAggMomentum : kAggSgd, ws, 0);
 }
 
 cudaError_t launch_list_tiles(const uint32_t* idx, const uint32_t* count, uint32_t d,

@@ -43,7 +43,7 @@ ef_status device_info(int dev, DeviceInfo* out) {
     ht_init_device(info);
     topk_init_device(info);
     topk_layerwise_init_device(info);
-    aggregate_init_device();
+    aggregate_init_device(info);
     if (info.refine_blocks <= 0 || info.finalize_blocks <= 0) return EF_ERR_CUDA;
     it = g_devices.emplace(dev, info).first;
   }
@@ -373,7 +373,8 @@ ef_status aggregate_entry(uint32_t n, const uint32_t* const* idx, const float* c
     return finish_launch(
         launch_aggregate_apply(n, idx, val, tiles, counts, d32, alpha, x, m, momentum, lr, *ws),
         ws);
-  return finish_launch(launch_aggregate(n, idx, val, tiles, counts, d32, dense_out, *ws), ws);
+  return finish_launch(launch_aggregate(n, idx, val, tiles, counts, d32, dense_out, *ws, info),
+                       ws);
 }
 
 }  // namespace efs

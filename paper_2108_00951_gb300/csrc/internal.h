@@ -205,6 +205,7 @@ struct DeviceInfo {
   int lw_group_per_sm_f32 = 0;    // layer-wise candidate pass, claimed-group kernel CTAs per SM
   int lw_group_per_sm_bf16 = 0;
   int lw_select_per_sm = 0;       // co-resident layer-wise select CTAs per SM
+  int agg_stream_slots = 0;       // resident CTAs of the persistent dense sum
 };
 
 // Per-device set-up of the Top-k kernels (shared-memory opt-in, occupancy).
@@ -215,7 +216,7 @@ void topk_layerwise_init_device(DeviceInfo& info);
 
 // Per-device set-up of the aggregation kernels (prefer the largest shared
 // memory carve-out, so that 8 of their CTAs are resident per SM).
-void aggregate_init_device();
+void aggregate_init_device(DeviceInfo& info);
 
 // Per-device set-up of the streaming hard-threshold kernels (opts them into
 // their shared-memory ring on the current device and records occupancy).
@@ -290,7 +291,7 @@ cudaError_t launch_topk_layerwise(const void* g, bool g_bf16, float* e, float ga
 // indexes; without it the kernel before the reduction finds them.
 cudaError_t launch_aggregate(uint32_t n, const uint32_t* const* idx, const float* const* val,
                              const uint32_t* const* tiles, const uint32_t* counts, uint32_t d,
-                             float* dense_out, Workspace& ws);
+                             float* dense_out, Workspace& ws, const DeviceInfo& dev);
 cudaError_t launch_aggregate_apply(uint32_t n, const uint32_t* const* idx,
                                    const float* const* val, const uint32_t* const* tiles,
                                    const uint32_t* counts, uint32_t d, float alpha, float* x,

@@ -1,0 +1,93 @@
+"""The dense sum's two kernels meet at 912 tiles, and its offsets come from a
+scatter or from searches: sizes on both sides, runs that fill a stage exactly,
+spill into a second one or fill a whole tile, 1 to 33 workers, lists that are
+not 16-byte aligned, and malformed lists, against the oracle."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import paper_2108_00951_gb300 as efs
+
+pytestmark = pytest.mark.gpu
+if not torch.cuda.is_available():
+    pytest.skip("needs a CUDA GPU", allow_module_level=True)
+
+import gpu_util as gu  # noqa: E402
+
+TILE = efs.TILE
+
+
+def _lists(d, counts, seed):
+    """Ascending lists, entries drawn evenly; with whole dense tiles and runs of
+    640 (a stage) and 641 pairs put into each."""
+    rng = np.random.default_rng(seed)
+    idx, val = [], []
+    for w, c in enumerate(counts):
+        j = rng.choice(d, c, replace=False)
+        t = 3 + 2 * w  # tiles with runs of 4096, 640 and 641 pairs
+        extra = [np.arange(t * TILE, (t + 1) * TILE),
+                 (t + 1) * TILE + np.sort(rng.choice(TILE, 640 + w % 2, replace=False))]
+        j = np.unique(np.concatenate([j] + (extra if c else [])))
+        idx.append(j.astype(np.uint32))
+        val.append((rng.standard_normal(j.size) * 10.0 ** rng.integers(-3, 3)).astype(np.float32))
+    return idx, val
+
+
+def _sum(idx, val, d, tiles, off=0):
+    it = [gu.to_dev(i.view(np.int32), off) if i.size else
+          torch.zeros(1, dtype=torch.int32, device=gu.DEV) for i in idx]
+    vt = [gu.to_dev(v, off) if v.size else torch.zeros(1, device=gu.DEV) for v in val]
+    counts = torch.tensor([i.size for i in idx], dtype=torch.int32, device=gu.DEV)
+    tt = None
+    if tiles:
+        edges = np.arange(efs.tiles_for(d) - 1, dtype=np.int64) * TILE
+        tt = [gu.to_dev(np.append(np.searchsorted(i.astype(np.int64), edges), i.size)
+                        .astype(np.int32)) for i in idx]
+    dense = torch.full((d,), float("nan"), device=gu.DEV)
+    efs.sparse_aggregate(it, vt, counts, d, dense, tiles=tt)
+    return dense.cpu().numpy()
+
+
+@pytest.mark.parametrize("off", [0, 1])
+@pytest.mark.parametrize("tiles", [False, True])
+@pytest.mark.parametrize("n", [1, 2, 16, 32, 33])
+@pytest.mark.parametrize("d", [911 * TILE, 911 * TILE + 1, 1300 * TILE - 5])
+def test_dense_sum_around_the_rule(d, n, tiles, off):
+    counts = [0 if w % 5 == 4 else 40 * 10 ** (w % 4) for w in range(n)]
+    idx, val = _lists(d, counts, n)
+    gu.assert_bits(_sum(idx, val, d, tiles, off), oracle.sparse_aggregate(idx, val, d),
+                   "d=%d n=%d tiles=%s off=%d" % (d, n, tiles, off))
+    assert efs.ef_check_status() == efs.EF_OK
+
+
+def test_more_entries_than_the_scatter_takes():
+    d, n = 1300 * TILE - 5, 3
+    idx, val = _lists(d, [3_000_000] * n, 9)  # over 8 M entries: searches
+    gu.assert_bits(_sum(idx, val, d, False), oracle.sparse_aggregate(idx, val, d), "long lists")
+    assert efs.ef_check_status() == efs.EF_OK
+
+
+def test_malformed_lists_many_tiles():
+    # a tile index that sends a tile another tile's pairs, and an index past d:
+    # skipped and latched, every other coordinate as if they were absent
+    d = 1000 * TILE
+    idx, val = _lists(d, [500, 500], 4)
+    edges = np.arange(1000, dtype=np.int64) * TILE
+    good = [np.append(np.searchsorted(i.astype(np.int64), edges), i.size) for i in idx]
+    wrong = good[1].copy()
+    wrong[10] = 0   # tile 10's run begins at the list's first pair
+    idx[0][-1] = d + 7
+    it = [gu.to_dev(i.view(np.int32)) for i in idx]
+    vt = [gu.to_dev(v) for v in val]
+    counts = torch.tensor([i.size for i in idx], dtype=torch.int32, device=gu.DEV)
+    tt = [gu.to_dev(t.astype(np.int32)) for t in (good[0], wrong)]
+    dense = torch.full((d,), float("nan"), device=gu.DEV)
+    efs.sparse_aggregate(it, vt, counts, d, dense, tiles=tt)
+    assert efs.ef_check_status() == efs.EF_ERR_BAD_INPUT
+    got = dense.cpu().numpy()
+    ref = oracle.sparse_aggregate([idx[0][:-1], idx[1]], [val[0][:-1], val[1]], d)
+    mask = np.ones(d, bool)
+    mask[9 * TILE:11 * TILE] = False   # tiles 9 and 10 got wrong runs
+    gu.assert_bits(got[mask], ref[mask], "untouched tiles")
+    assert np.all(np.isfinite(got))
