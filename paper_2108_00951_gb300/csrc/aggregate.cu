@@ -32,10 +32,15 @@
 namespace efs {
 namespace {
 
+// The lists, passed as kernel parameters: 768 bytes for up to 32 workers, 6 KB
+// for more (a launch copies its parameters: an exchange of 4 lists took the
+// host 5.3 us with the large form).
+constexpr uint32_t kFewWorkers = 32;
+template <uint32_t kCap>
 struct AggPtrs {
-  const uint32_t* idx[kMaxWorkers];
-  const float* val[kMaxWorkers];
-  const uint32_t* tiles[kMaxWorkers];  // the lists' tile indexes, when the caller has them
+  const uint32_t* idx[kCap];
+  const float* val[kCap];
+  const uint32_t* tiles[kCap];  // the lists' tile indexes, when the caller has them
 };
 
 // off[i * (tiles + 1) + t] = number of entries of list i below t * kAggTile;
@@ -58,8 +63,9 @@ struct AggPtrs {
 // LSTM-shaped workers' steps with their exchange (0.9 M entries each) 333.5 ->
 // 300.2.
 constexpr uint32_t kScatterEntries = 8u << 20;
+template <uint32_t kCap>
 __global__ void __launch_bounds__(kThreads)
-    agg_offsets_kernel(AggPtrs p, const uint32_t* __restrict__ counts, uint32_t n,
+    agg_offsets_kernel(AggPtrs<kCap> p, const uint32_t* __restrict__ counts, uint32_t n,
                        uint32_t tiles, uint32_t* __restrict__ off, uint32_t* __restrict__ error) {
   griddep_wait();                // the lists and counts come from the kernels before
   griddep_launch_dependents();    // the reduction may be scheduled (it waits for this grid)
@@ -174,13 +180,13 @@ __device__ __forceinline__ void prefetch_l2_bulk(const void* p, uint32_t bytes) 
   asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
 }
 
-template <bool kVec, int kMode>
+template <bool kVec, int kMode, uint32_t kCap>
 __global__ void __launch_bounds__(kThreads)
-    agg_reduce_kernel(AggPtrs p, uint32_t n, uint32_t d, uint32_t tiles,
+    agg_reduce_kernel(AggPtrs<kCap> p, uint32_t n, uint32_t d, uint32_t tiles,
                       const uint32_t* __restrict__ off, const uint32_t* __restrict__ counts,
                       AggOut o, uint32_t* __restrict__ error) {
   __shared__ __align__(16) float acc[kAggTile];
-  __shared__ uint32_t s_lo[kMaxWorkers], s_pre[kMaxWorkers + 1];
+  __shared__ uint32_t s_lo[kCap], s_pre[kCap + 1];
   __shared__ uint32_t st_idx[kAggStage];
   __shared__ float st_val[kAggStage];
   const uint32_t t = blockIdx.x;
@@ -341,7 +347,7 @@ static_assert(offsetof(AggStream, idx) % 16 == 0 && offsetof(AggStream, val) % 1
 
 template <bool kVec>
 __global__ void __launch_bounds__(32)
-    agg_stream_kernel(AggPtrs p, uint32_t n, uint32_t d, uint32_t tiles,
+    agg_stream_kernel(AggPtrs<kFewWorkers> p, uint32_t n, uint32_t d, uint32_t tiles,
                       const uint32_t* __restrict__ off, const uint32_t* __restrict__ counts,
                       float* __restrict__ out, uint32_t* __restrict__ error,
                       uint64_t wait_limit_ns) {
@@ -550,66 +556,98 @@ __global__ void __launch_bounds__(32)
   if (bad) atomicOr(error, kDevErrBadInput);
 }
 
-template <int kMode>
-cudaError_t launch_reduce(bool vec, AggPtrs p, uint32_t n, uint32_t d, uint32_t tiles,
+template <int kMode, uint32_t kCap>
+cudaError_t launch_reduce(bool vec, AggPtrs<kCap>& p, uint32_t n, uint32_t d, uint32_t tiles,
                           const uint32_t* off, const uint32_t* counts, AggOut o, Workspace& ws) {
   uint32_t* error = ws.u32(kOffError);
   void* params[] = {&p, &n, &d, &tiles, &off, &counts, &o, &error};
-  const void* fn = vec ? reinterpret_cast<const void*>(&agg_reduce_kernel<true, kMode>)
-                       : reinterpret_cast<const void*>(&agg_reduce_kernel<false, kMode>);
+  const void* fn = vec ? reinterpret_cast<const void*>(&agg_reduce_kernel<true, kMode, kCap>)
+                       : reinterpret_cast<const void*>(&agg_reduce_kernel<false, kMode, kCap>);
   return launch_pdl(fn, tiles, kThreads, 0, ws.stream, params, false);
 }
 
+// Each list's position at every tile boundary, for lists without tile indexes.
+template <uint32_t kCap>
+cudaError_t launch_offsets(AggPtrs<kCap>& p, const uint32_t* counts, uint32_t n, uint32_t tiles,
+                           uint32_t* off, Workspace& ws) {
+  // a thread per tile for the searches; for the scatter about 8 CTAs per SM
+  // in all, but no more than 16 entries a tile would occupy
+  const uint32_t per_tile = (tiles + 1 + kThreads - 1) / kThreads;
+  const uint32_t wide = std::min((1216 + n - 1) / n, (tiles / kThreads + 1) * 16);
+  const dim3 grid(std::max(per_tile, wide), n);
+  uint32_t* error = ws.u32(kOffError);
+  void* params[] = {&p, &counts, &n, &tiles, &off, &error};
+  const cudaError_t err = launch_pdl(reinterpret_cast<const void*>(&agg_offsets_kernel<kCap>),
+                                     grid, kThreads, 0, ws.stream, params, false);
+  count_launch();
+  return err;
+}
+
+template <uint32_t kCap>
 cudaError_t launch_common(uint32_t n, const uint32_t* const* idx, const float* const* val,
                           const uint32_t* const* tile_index, const uint32_t* counts, uint32_t d,
                           const AggOut& o, int mode, Workspace& ws, int agg_stream_slots) {
-  AggPtrs p;
-  for (uint32_t i = 0; i < kMaxWorkers; ++i) {
-    p.idx[i] = i < n ? idx[i] : nullptr;
-    p.val[i] = i < n ? val[i] : nullptr;
-    p.tiles[i] = i < n && tile_index ? tile_index[i] : nullptr;
+  AggPtrs<kCap> p;
+  for (uint32_t i = 0; i < n; ++i) {
+    p.idx[i] = idx[i];
+    p.val[i] = val[i];
+    p.tiles[i] = tile_index ? tile_index[i] : nullptr;
   }
-  const uint32_t tiles = agg_tiles_for(d);
+  uint32_t tiles = agg_tiles_for(d);
   cudaError_t err = cudaSuccess;
   uint32_t* off = nullptr;
   if (!tile_index) {  // locate each list's tile boundaries first
-    // a thread per tile for the searches; for the scatter about 8 CTAs per SM
-    // in all, but no more than 16 entries a tile would occupy
-    const uint32_t per_tile = (tiles + 1 + kThreads - 1) / kThreads;
-    const uint32_t wide = std::min((1216 + n - 1) / n, (tiles / kThreads + 1) * 16);
-    const dim3 grid1(std::max(per_tile, wide), n);
     off = ws.offsets();
-    const uint32_t* counts_arg = counts;
-    uint32_t n_arg = n, tiles_arg = tiles;
-    uint32_t* error = ws.u32(kOffError);
-    void* params[] = {&p, &counts_arg, &n_arg, &tiles_arg, &off, &error};
-    err = launch_pdl(reinterpret_cast<const void*>(&agg_offsets_kernel), grid1, kThreads, 0,
-                     ws.stream, params, false);
-    count_launch();
+    err = launch_offsets(p, counts, n, tiles, off, ws);
     if (err != cudaSuccess) return err;
   }
   const bool vec = reinterpret_cast<uintptr_t>(o.out) % 16 == 0 &&
                    reinterpret_cast<uintptr_t>(o.m) % 16 == 0;
-  if (mode == kAggDense && n <= 32 && tiles >= kAggMinTiles && agg_stream_slots > 0) {
-    uint32_t n_arg = n, tiles_arg = tiles;
-    const uint32_t* counts_arg = counts;
-    float* out = o.out;
-    uint32_t* error = ws.u32(kOffError);
-    uint64_t limit = wait_limit_ns();
-    void* params[] = {&p, &n_arg, &d, &tiles_arg, &off, &counts_arg, &out, &error, &limit};
-    const void* fn = vec ? reinterpret_cast<const void*>(&agg_stream_kernel<true>)
-                         : reinterpret_cast<const void*>(&agg_stream_kernel<false>);
-    const uint32_t slots = static_cast<uint32_t>(agg_stream_slots);
-    err = launch_pdl(fn, tiles < slots ? tiles : slots, 32, sizeof(AggStream), ws.stream, params,
-                     false);
-  } else if (mode == kAggDense)
+  if (mode == kAggDense) {
+    if constexpr (kCap == kFewWorkers) {
+      if (tiles >= kAggMinTiles && agg_stream_slots > 0) {
+        float* out = o.out;
+        uint32_t* error = ws.u32(kOffError);
+        uint64_t limit = wait_limit_ns();
+        void* params[] = {&p, &n, &d, &tiles, &off, &counts, &out, &error, &limit};
+        const void* fn = vec ? reinterpret_cast<const void*>(&agg_stream_kernel<true>)
+                             : reinterpret_cast<const void*>(&agg_stream_kernel<false>);
+        err = launch_pdl(fn, std::min(tiles, static_cast<uint32_t>(agg_stream_slots)), 32,
+                         sizeof(AggStream), ws.stream, params, false);
+        count_launch();
+        return err;
+      }
+    }
     err = launch_reduce<kAggDense>(vec, p, n, d, tiles, off, counts, o, ws);
-  else if (mode == kAggSgd)
+  } else if (mode == kAggSgd) {
     err = launch_reduce<kAggSgd>(vec, p, n, d, tiles, off, counts, o, ws);
-  else
+  } else {
     err = launch_reduce<kAggMomentum>(vec, p, n, d, tiles, off, counts, o, ws);
+  }
   count_launch();
   return err;
+}
+
+cudaError_t launch_any(uint32_t n, const uint32_t* const* idx, const float* const* val,
+                       const uint32_t* const* tiles, const uint32_t* counts, uint32_t d,
+                       const AggOut& o, int mode, Workspace& ws, int agg_stream_slots) {
+  return n <= kFewWorkers ? launch_common<kFewWorkers>(n, idx, val, tiles, counts, d, o, mode, ws,
+                                                       agg_stream_slots)
+                          : launch_common<kMaxWorkers>(n, idx, val, tiles, counts, d, o, mode, ws,
+                                                       agg_stream_slots);
+}
+
+template <uint32_t kCap>
+void prefer_shared() {
+  const void* fns[] = {reinterpret_cast<const void*>(&agg_reduce_kernel<true, kAggDense, kCap>),
+                       reinterpret_cast<const void*>(&agg_reduce_kernel<false, kAggDense, kCap>),
+                       reinterpret_cast<const void*>(&agg_reduce_kernel<true, kAggSgd, kCap>),
+                       reinterpret_cast<const void*>(&agg_reduce_kernel<false, kAggSgd, kCap>),
+                       reinterpret_cast<const void*>(&agg_reduce_kernel<true, kAggMomentum, kCap>),
+                       reinterpret_cast<const void*>(&agg_reduce_kernel<false, kAggMomentum, kCap>)};
+  for (const void* f : fns)
+    cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout,
+                         cudaSharedmemCarveoutMaxShared);
 }
 }  // namespace
 
@@ -628,23 +666,15 @@ void aggregate_init_device(DeviceInfo& info) {
     per_sm = f == streams[0] || b < per_sm ? b : per_sm;
   }
   info.agg_stream_slots = per_sm * info.sm_count;
-  const void* fns[] = {
-      reinterpret_cast<const void*>(&agg_reduce_kernel<true, kAggDense>),
-      reinterpret_cast<const void*>(&agg_reduce_kernel<false, kAggDense>),
-      reinterpret_cast<const void*>(&agg_reduce_kernel<true, kAggSgd>),
-      reinterpret_cast<const void*>(&agg_reduce_kernel<false, kAggSgd>),
-      reinterpret_cast<const void*>(&agg_reduce_kernel<true, kAggMomentum>),
-      reinterpret_cast<const void*>(&agg_reduce_kernel<false, kAggMomentum>)};
-  for (const void* f : fns)
-    cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout,
-                         cudaSharedmemCarveoutMaxShared);
+  prefer_shared<kFewWorkers>();
+  prefer_shared<kMaxWorkers>();
   cudaGetLastError();
 }
 
 cudaError_t launch_aggregate(uint32_t n, const uint32_t* const* idx, const float* const* val,
                              const uint32_t* const* tiles, const uint32_t* counts, uint32_t d,
                              float* dense_out, Workspace& ws, const DeviceInfo& dev) {
-  return launch_common(n, idx, val, tiles, counts, d,
+  return launch_any(n, idx, val, tiles, counts, d,
                        AggOut{dense_out, nullptr, 1.0f, 0.0f, 0.0f}, kAggDense, ws,
                        dev.agg_stream_slots);
 }
@@ -653,26 +683,15 @@ cudaError_t launch_aggregate_apply(uint32_t n, const uint32_t* const* idx,
                                    const float* const* val, const uint32_t* const* tiles,
                                    const uint32_t* counts, uint32_t d, float alpha, float* x,
                                    float* m, float mu, float lr, Workspace& ws) {
-  return launch_common(n, idx, val, tiles, counts, d, AggOut{x, m, alpha, mu, lr},
+  return launch_any(n, idx, val, tiles, counts, d, AggOut{x, m, alpha, mu, lr},
                        m ? kAggMomentum : kAggSgd, ws, 0);
 }
 
 cudaError_t launch_list_tiles(const uint32_t* idx, const uint32_t* count, uint32_t d,
                               uint32_t* tiles_out, Workspace& ws) {
-  AggPtrs p;
-  for (uint32_t i = 0; i < kMaxWorkers; ++i) {
-    p.idx[i] = i == 0 ? idx : nullptr;
-    p.val[i] = nullptr;
-    p.tiles[i] = nullptr;
-  }
-  uint32_t n = 1, tiles = agg_tiles_for(d);
-  const dim3 grid((tiles + 1 + kThreads - 1) / kThreads, 1);
-  uint32_t* error = ws.u32(kOffError);
-  void* params[] = {&p, &count, &n, &tiles, &tiles_out, &error};
-  const cudaError_t err = launch_pdl(reinterpret_cast<const void*>(&agg_offsets_kernel), grid,
-                                     kThreads, 0, ws.stream, params, false);
-  count_launch();
-  return err;
+  AggPtrs<kFewWorkers> p;
+  p.idx[0] = idx;
+  return launch_offsets(p, count, 1, agg_tiles_for(d), tiles_out, ws);
 }
 
 }  // namespace efs
