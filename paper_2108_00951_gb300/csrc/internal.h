@@ -37,7 +37,9 @@ constexpr int kHistBins = 2048;
 constexpr int kSampleBits = 13;         // the sample histogram: top 13 bits of |a|
 constexpr int kSampleBins = 1 << kSampleBits;
 constexpr size_t kStSampleHist = kStHist + sizeof(uint32_t) * kHistLevels * kHistBins;
-constexpr size_t kTkStateBytes = kStSampleHist + sizeof(uint32_t) * kSampleBins;
+constexpr size_t kStWindowHist = kStSampleHist + sizeof(uint32_t) * kSampleBins;
+                                        // uint32[2048]: the on-chip select's histogram
+constexpr size_t kTkStateBytes = kStWindowHist + sizeof(uint32_t) * kHistBins;
 static_assert(kTkStateBytes % 256 == 0, "state block alignment");
 constexpr size_t kHeaderBytes = kOffTkState + 2 * kTkStateBytes;
 constexpr uint32_t kMaxChunks = 1024;   // per-CTA chunk sums of the streaming compaction

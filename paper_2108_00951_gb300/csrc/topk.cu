@@ -29,9 +29,10 @@
 //             e at the selected coordinates. Up to 48 K candidates CTA 0
 //             finds the threshold in shared memory (digit levels over the
 //             candidates' own magnitude range) and slice CTAs write the pairs
-//             in parallel; beyond, the whole grid runs a radix select (merged
-//             histograms with bounded grid barriers; chunk counts, then
-//             positions).
+//             in parallel. Beyond, while the grid's shared memory holds the
+//             list, every CTA keeps its slice on chip (onchip_select); else
+//             the whole grid runs a radix select (merged histograms with
+//             bounded grid barriers; chunk counts, then positions).
 // The candidate path moves about 12 B per coordinate plus small amounts; the
 // full-array path adds a read of a per digit level and two for the output.
 #include <algorithm>
@@ -56,7 +57,8 @@ __device__ __forceinline__ uint64_t composite_key(float a, uint64_t j) {
 }
 
 struct TopkArgs {
-  uint32_t* hist;        // [kHistLevels + 1][kHistBins]
+  uint32_t* hist;        // [kHistLevels][kHistBins]
+  uint32_t* window_hist; // [kHistBins], the on-chip select's
   uint64_t* cand0;       // key buffers of the refine levels
   uint64_t* cand1;
   uint32_t* list_idx;    // ordered candidates from the streaming pass
@@ -74,6 +76,7 @@ struct TopkArgs {
   uint64_t* chunk_sums;
   uint32_t epoch;        // tags the finalize kernel's chunk totals
   uint64_t wait_limit_ns;
+  uint32_t* err_arrive;  // CTAs of the on-chip select that published their share (zero at start)
   double* err_out;       // optional ||e'||^2 of the step
   const double* stream_err;  // the streaming pass's share (coordinates below the bound)
   FF* err_parts;         // [gridDim.x] the select CTAs' shares
@@ -130,9 +133,15 @@ struct TopkCandOp : StreamIn<GT, kAny> {
       x[2] = __fmaf_rn(gamma, gv[2], ev.z);
       x[3] = __fmaf_rn(gamma, gv[3], ev.w);
     }
+    // plain atomics (warp-aggregated ones take longer), zeros by the warp
+    // together: a vector's exact zeros would all meet in one bin
 #pragma unroll
-    for (int j = 0; j < 4; ++j)
-      hist_add_warp(s_hist, (__float_as_uint(x[j]) & 0x7fffffffu) >> kSampleShift, in);
+    for (int j = 0; j < 4; ++j) {
+      const uint32_t bin = (__float_as_uint(x[j]) & 0x7fffffffu) >> kSampleShift;
+      const uint32_t zeros = __ballot_sync(0xffffffffu, in && bin == 0);
+      if (in && bin) atomicAdd(&s_hist[bin], 1u);
+      if ((threadIdx.x & 31) == 0 && zeros) atomicAdd(&s_hist[0], __popc(zeros));
+    }
   }
 
   __device__ void merge(const uint32_t* s_hist) const {
@@ -593,6 +602,217 @@ __device__ void small_emit(const TopkArgs& args, float* e, uint32_t n, uint32_t 
   if (__syncthreads_or(overflow) && tid == 0) atomicOr(args.error, kDevErrOverflow);
 }
 
+// A list beyond one CTA's shared memory that the grid's shared memory holds:
+// each CTA keeps its slice (values and coordinates) on chip and reads it from
+// L2 once.
+//  1 Every CTA histograms its slice over one binade from the candidate bound
+//    up, in 2048 windows of 4096 magnitude patterns (larger magnitudes in the
+//    last); the merged histogram, behind a grid barrier, gives the window
+//    with the k-th magnitude.
+//  2 Every CTA counts its magnitudes above the window and copies those in it,
+//    in list order, to its region in global memory; behind a second grid
+//    barrier every CTA reads all of them (about n / 2048, so a few thousand)
+//    into one ordered list and finds the exact threshold there, ties by
+//    position; its output position follows from the same counts.
+//  3 It writes its selected pairs in order and zeroes e at each.
+// The slices cost one round trip and the barriers two; the radix select below
+// reads the list five times around three to six barriers. Measured on a
+// GB300, LSTM-shaped call, k = 289 K of 28.9 M (0.45 M candidates): this
+// kernel 45 -> 28 us, the call 123 -> 103.5; ResNet-50-shaped, k = 1 %, 117 ->
+// 97; VGG-16-shaped, k = 1 %, 428 -> 358. Lists that one CTA holds stay with
+// it (ResNet-18-shaped, k = 0.1 %, 17 K candidates: 47.5 us a call, 57.8 this
+// way): its few CTAs let the next call's sampling start beside them. Returns false, uniformly over the grid, when it does not apply
+// (the k-th magnitude more than a binade above the bound, or too many
+// magnitudes in its window); the radix select then runs.
+constexpr uint32_t kSliceCap = 16384;   // pairs of a slice in shared memory
+constexpr uint32_t kGatherCap = 12288;  // magnitudes of the k-th one's window
+constexpr uint32_t kRegionCap = 1024;   // those of one CTA
+constexpr int kWindowShift = 12;        // log2 of the magnitudes per window
+static_assert(2 * kSliceCap + kGatherCap + 1024 <= kSmallCand, "on-chip select's shared memory");
+
+__device__ bool onchip_select(const TopkArgs& args, float* e, uint32_t n, uint32_t k,
+                              uint32_t* smem, uint32_t* s_hist, uint32_t* s_w, uint32_t* idx_out,
+                              float* val_out, uint32_t* count_out) {
+  const uint32_t G = gridDim.x, c = blockIdx.x, tid = threadIdx.x;
+  const uint32_t lo = static_cast<uint32_t>(static_cast<uint64_t>(c) * n / G);
+  const uint32_t m = static_cast<uint32_t>(static_cast<uint64_t>(c + 1) * n / G) - lo;
+  uint32_t* const s_val = smem;              // value bits of the slice
+  uint32_t* const s_idx = smem + kSliceCap;  // and coordinates
+  uint32_t* const s_mags = s_idx + kSliceCap;  // the window's magnitudes, all CTAs'
+  uint32_t* const s_pre = s_mags + kGatherCap; // where each CTA's begin
+  constexpr uint32_t kBlock = 4 * kSelThreads;  // positions per ordered round
+
+  // 1 the slice, and its histogram
+  for (uint32_t b = tid; b < static_cast<uint32_t>(kHistBins); b += kSelThreads) s_hist[b] = 0;
+  for (uint32_t i0 = tid; i0 < m; i0 += 4 * kSelThreads) {
+    uint32_t v[4], x[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {  // all loads in flight together
+      const uint32_t i = i0 + j * kSelThreads;
+      v[j] = i < m ? __float_as_uint(__ldcg(args.list_val + lo + i)) : 0u;
+      x[j] = i < m ? __ldcg(args.list_idx + lo + i) : 0u;
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const uint32_t i = i0 + j * kSelThreads;
+      if (i < m) {
+        s_val[i] = v[j];
+        s_idx[i] = x[j];
+      }
+    }
+  }
+  const uint32_t bound = static_cast<uint32_t>(__ldcg(args.lower_bound) >> 32);
+  __syncthreads();
+  for (uint32_t i = tid; i < m; i += kSelThreads)
+    atomicAdd(&s_hist[min(((s_val[i] & 0x7fffffffu) - bound) >> kWindowShift, kHistBins - 1u)],
+              1u);
+  __syncthreads();
+  for (uint32_t b = tid; b < static_cast<uint32_t>(kHistBins); b += kSelThreads)
+    if (s_hist[b]) atomicAdd(&args.window_hist[b], s_hist[b]);
+  if (!grid_barrier(args.bar_arrive, args.bar_gen, args.wait_limit_ns, args.error)) return false;
+  const Selection s = select_bin<kSelThreads, true>(args.window_hist, kHistBins, k, s_w);
+  if (!s.found || s.bin == kHistBins - 1 || s.n_in > kGatherCap) return false;
+  const uint32_t w0 = bound + (s.bin << kWindowShift), width = 1u << kWindowShift;
+
+  // 2 the window's magnitudes
+  const uint32_t cap = min(kRegionCap, args.cand_cap / G * 2 - 2);  // 4-byte words of cand0
+  uint32_t* const region = reinterpret_cast<uint32_t*>(args.cand0) + static_cast<size_t>(c) * (cap + 2);
+  uint32_t n_in = 0, n_above = 0;
+  for (uint32_t b0 = 0; b0 < m; b0 += kBlock) {
+    uint32_t mag[4], in = 0, above = 0;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const uint32_t i = b0 + 4 * tid + j;
+      mag[j] = i < m ? s_val[i] & 0x7fffffffu : 0u;
+      in |= (mag[j] - w0 < width ? 1u : 0u) << j;
+      above += mag[j] >= w0 + width ? 1u : 0u;
+    }
+    uint32_t total;
+    uint32_t at = n_in + (block_exclusive<kSelThreads>((__popc(in) << 16) | above, total, s_w) >> 16);
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      if (in & (1u << j)) {
+        if (at < cap) region[2 + at] = mag[j];
+        ++at;
+      }
+    n_in += total >> 16;
+    n_above += total & 0xffffu;
+  }
+  if (tid == 0) {
+    region[0] = n_in;
+    region[1] = n_above;
+  }
+  if (!grid_barrier(args.bar_arrive, args.bar_gen, args.wait_limit_ns, args.error)) return false;
+  const uint32_t* const regions = reinterpret_cast<const uint32_t*>(args.cand0);
+  uint32_t their_in = 0, their_above = 0;
+  if (tid < G) {
+    their_in = __ldcg(regions + static_cast<size_t>(tid) * (cap + 2));
+    their_above = __ldcg(regions + static_cast<size_t>(tid) * (cap + 2) + 1);
+  }
+  uint32_t all_in, ignored;
+  const uint32_t before_in = block_exclusive<kSelThreads>(their_in, all_in, s_w);
+  const uint32_t before_above = block_exclusive<kSelThreads>(their_above, ignored, s_w);
+  __shared__ uint32_t s_my_above;
+  s_pre[tid] = before_in;  // for tid >= G: the end
+  if (tid == c) s_my_above = before_above;
+  if (__syncthreads_or(their_in > cap) || all_in != s.n_in) return false;
+  for (uint32_t i = tid; i < all_in; i += kSelThreads) {
+    uint32_t a = 0, z = G;  // the CTA whose magnitudes reach past i
+    while (z - a > 1) {
+      const uint32_t h = (a + z) / 2;
+      if (s_pre[h] <= i) a = h;
+      else z = h;
+    }
+    s_mags[i] = __ldcg(regions + static_cast<size_t>(a) * (cap + 2) + 2 + (i - s_pre[a]));
+  }
+  __syncthreads();
+  SmallSelection sel;
+  if (!threshold_levels<kSelThreads>(MagsShared{s_mags}, all_in, s.k_rem, w0, w0 + width - 1,
+                                     s_hist, s_w, sel))
+    return false;
+  // the pairs of earlier CTAs, and how many of this one's equal magnitudes are taken
+  uint32_t earlier = 0, equal = 0;
+  const uint32_t my_end = s_pre[c] + n_in;
+  for (uint32_t i = tid; i < my_end; i += kSelThreads) {
+    const uint32_t mg = s_mags[i];
+    if (i < s_pre[c])
+      earlier += selected(sel, mg, i) ? 1u : 0u;
+    else
+      equal += mg == sel.B && i <= sel.last ? 1u : 0u;
+  }
+  uint32_t sum_earlier, quota;
+  block_exclusive<kSelThreads>(earlier, sum_earlier, s_w);
+  block_exclusive<kSelThreads>(equal, quota, s_w);
+
+  // 3 the pairs
+  uint32_t base = s_my_above + sum_earlier, eq_seen = 0;
+  bool overflow = false;
+  ErrAcc acc;
+  for (uint32_t b0 = 0; b0 < m; b0 += kBlock) {
+    const uint32_t i0 = b0 + 4 * tid;
+    uint32_t v[4], eq = 0, take = 0;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      v[j] = i0 + j < m ? s_val[i0 + j] : 0u;
+      const uint32_t mg = v[j] & 0x7fffffffu;
+      if (i0 + j < m) {
+        take |= (mg > sel.B ? 1u : 0u) << j;
+        eq |= (mg == sel.B ? 1u : 0u) << j;
+      }
+    }
+    uint32_t total;
+    if (sel.ties) {
+      uint32_t rank = eq_seen + block_exclusive<kSelThreads>(__popc(eq), total, s_w);
+      eq_seen += total;
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        if ((eq >> j) & 1u) take |= (rank++ < quota ? 1u : 0u) << j;
+    } else {
+      take |= eq;
+    }
+    uint32_t pos = base + block_exclusive<kSelThreads>(__popc(take), total, s_w);
+    base += total;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      if ((take >> j) & 1u) {
+        if (pos < k) {
+          const uint32_t x = s_idx[i0 + j];
+          idx_out[pos] = x;
+          val_out[pos] = __uint_as_float(v[j]);
+          e[x] = 0.0f;  // residual of a sent coordinate
+        } else {
+          overflow = true;
+        }
+        ++pos;
+      } else if (args.err_out && i0 + j < m) {
+        acc.add(__uint_as_float(v[j]));
+      }
+    }
+  }
+  if (c == G - 1 && tid == 0) *count_out = base < k ? base : k;
+  if (__syncthreads_or(overflow) && tid == 0) atomicOr(args.error, kDevErrOverflow);
+  if (args.err_out) {
+    // the candidates not sent keep a; the last CTA adds the shares in CTA
+    // order to the streaming pass's
+    __shared__ FF s_d[32];
+    __shared__ uint32_t s_last_cta;
+    acc.flush();
+    const FF share = block_sum_ff(acc.total, s_d);
+    if (tid == 0) {
+      args.err_parts[c] = share;
+      __threadfence();
+      s_last_cta = atomicAdd(args.err_arrive, 1u) == G - 1 ? 1u : 0u;
+    }
+    __syncthreads();
+    if (s_last_cta) {
+      __threadfence();
+      const FF shares = sum_parts_ff(args.err_parts, G, s_d);
+      if (tid == 0) *args.err_out = *args.stream_err + ff_to_double(shares);
+    }
+  }
+  return true;
+}
+
 // Radix select of the k-th largest composite key of the source across the
 // grid: merged global histograms, bounded grid barriers, candidate compaction
 // into key buffers once a bucket fits.
@@ -726,6 +946,9 @@ __global__ void __launch_bounds__(kSelThreads, 1)
     small_emit(args, e, si.n, k, Gs, idx_out, val_out, count_out, s_w);
     return;
   }
+  if (si.mode == 0 && static_cast<uint64_t>(si.n) <= static_cast<uint64_t>(gridDim.x) * kSliceCap &&
+      onchip_select(args, e, si.n, k, s_mag, s_hist, s_w, idx_out, val_out, count_out))
+    return;
   bool ok = true;
   const uint64_t thr = radix_threshold_grid(args, e, si, k, s_hist, s_w, ok);
   if (!ok) {
@@ -858,6 +1081,8 @@ cudaError_t launch_typed(const GT* g, float* e, float gamma, uint32_t k, uint32_
 
   TopkArgs args;
   args.hist = state + kStHist / 4;
+  args.window_hist = state + kStWindowHist / 4;
+  args.err_arrive = state + kStErrArrive / 4;
   args.cand0 = ws.cand(1);
   args.cand1 = ws.cand(2);
   args.list_idx = reinterpret_cast<uint32_t*>(ws.cand(0));
