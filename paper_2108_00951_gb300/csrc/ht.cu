@@ -166,8 +166,12 @@ struct HtOp : StreamIn<GT, kAny> {
 template <typename GT>
 constexpr int kHtStages = sizeof(GT) == 2 ? 5 : 4;
 
+// group entries: the shallow ring is the dense calls'
+template <typename GT, int kStages>
+constexpr int kHtEntries = kStages < kHtStages<GT> ? kLbFewEntries : kLbManyEntries;
+
 template <typename GT, bool kAny, int kStages = kHtStages<GT>>
-using HtGroupKernel = LbLayout<HtOp<GT, kAny>, kStages>;
+using HtGroupKernel = LbLayout<HtOp<GT, kAny>, kStages, kHtEntries<GT, kStages>>;
 template <typename GT, bool kAny>
 using HtChunkKernel = StreamLayout<HtOp<GT, kAny>, kHtStages<GT>>;
 
@@ -190,12 +194,12 @@ cudaError_t launch_groups(const StreamIn<GT, kAny>& in, float gamma, float lambd
   uint32_t cap = d;
   ScanCtx c = ctx;
   // the groups' shares of ||e'||^2 use the per-tile count area (16 words a tile)
-  LbArgs la{tiles_out, err_out, reinterpret_cast<FF*>(ws.counts()), ws.stage_idx(),
-            ws.stage_val(), ws.density_dev};
+  LbArgs la{tiles_out, err_out, reinterpret_cast<FF*>(ws.counts()), ws.stage_pairs(), ws.density_dev};
   void* params[] = {&op, &idx_out, &val_out, &count_out, &cap, &c, &la};
   const cudaError_t err = launch_pdl(
-      reinterpret_cast<const void*>(&lookback_stream_kernel<HtOp<GT, kAny>, kStages>), grid,
-      kLbThreads, HtGroupKernel<GT, kAny, kStages>::kSmem, ws.stream, params, false);
+      reinterpret_cast<const void*>(
+          &lookback_stream_kernel<HtOp<GT, kAny>, kStages, kHtEntries<GT, kStages>>),
+      grid, kLbThreads, HtGroupKernel<GT, kAny, kStages>::kSmem, ws.stream, params, false);
   count_launch();
   ws.ht_part_ready = false;  // the chunk kernel's boundaries are not written by this kernel
   return err;
@@ -295,7 +299,9 @@ int blocks_per_sm(const void* fn, int threads) {
 template <typename GT, bool kAny, int kStages>
 int group_blocks() {
   return blocks_per_sm<GT, HtGroupKernel<GT, kAny, kStages>>(
-      reinterpret_cast<const void*>(&lookback_stream_kernel<HtOp<GT, kAny>, kStages>), kLbThreads);
+      reinterpret_cast<const void*>(
+          &lookback_stream_kernel<HtOp<GT, kAny>, kStages, kHtEntries<GT, kStages>>),
+      kLbThreads);
 }
 template <typename GT, int kStages>
 int group_blocks_per_sm() {

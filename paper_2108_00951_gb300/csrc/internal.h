@@ -180,6 +180,8 @@ struct Workspace {
   float* stage_val() const {
     return reinterpret_cast<float*>(base + off_stage() + sizeof(uint32_t) * stage_cap);
   }
+  // the same area as (index, value bits) pairs: the claimed-group kernel's slots
+  uint2* stage_pairs() const { return reinterpret_cast<uint2*>(base + off_stage()); }
   uint32_t* u32(size_t off) const { return reinterpret_cast<uint32_t*>(base + off); }
   uint32_t* topk_state(uint32_t parity) const {
     return u32(kOffTkState + (parity & 1u) * kTkStateBytes);

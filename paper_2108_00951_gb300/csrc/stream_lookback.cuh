@@ -12,7 +12,8 @@
 // only ever waits for groups claimed before it (held by CTAs that are
 // already running), progress does not depend on which CTAs are resident.
 //
-// Roles (warps of a CTA):
+// Roles (warps of a CTA), which hand groups to one another through a ring of
+// entries with three mbarriers each (counted, ready, free):
 //  - 16 compute warps. Warp w owns the 256-coordinate segment [w*256,
 //    (w+1)*256) of every tile (the element layout of stream_compact.cuh). A
 //    group's two tiles arrive in consecutive ring stages; the warp computes
@@ -20,22 +21,33 @@
 //    then, once for the group: the positions of its selected pairs (one warp
 //    scan of the four units' counts), the pairs appended to its own circular
 //    buffer in shared memory — or, for a segment that finds no room, to the
-//    segment's slot in global memory —, the counts recorded in the group's
-//    entry. The warp that completes a group publishes its aggregate.
+//    segment's slot in global memory —, and for each segment a word with its
+//    count and place in the group's entry; its arrival on "counted" is all
+//    that the others need of it.
 //  - a producer warp: lane 1 claims groups, up to kLbClaimAhead ahead; lane 0
 //    takes a claimed group when an entry is free and issues the bulk copies
 //    (cp.async.bulk, completing on the stage's "full" mbarrier) of its tiles
 //    as ring stages are released; after the last group, an end marker.
-//  - a look-back warp: for each group of the CTA in claim order, the
+//  - an aggregate warp publishes each counted group's total.
+//  - a look-back warp: for each counted group of the CTA in claim order, the
 //    decoupled look-back over the published group totals (Merrill & Garland,
 //    the routine of the one-tile-per-CTA kernel), the inclusive total
 //    published, then the output position of each of the group's segments in
-//    (tile, warp) order, which is coordinate order.
-//  - kLbPlaceWarps placer warps: for each group, once its positions are
-//    there, they copy its segments (placer p: segments p, p + kLbPlaceWarps,
-//    ...; a warp's lanes on consecutive pairs, so loads and stores are
-//    coalesced) from the buffers or slots to the output, then hand the
-//    buffers' space back and free the entry.
+//    (tile, warp) order, which is coordinate order; arrives on "ready".
+//  - kLbPlaceWarps placer warps: for each ready group, placer p copies the
+//    segments p, p + kLbPlaceWarps, ... (a warp's lanes on consecutive pairs,
+//    so loads and stores are coalesced) from the buffers or slots to the
+//    output; the last to finish a group hands the buffers' space back and
+//    frees the entry.
+// A warp that waits is suspended on an mbarrier and issues next to nothing:
+// the compute warps, whose instruction chain bounds the kernel, have the
+// issue slots. Measured on a GB300, us a call, against the same roles with
+// polled words, a counter that the compute warps increment, and a barrier of
+// all placers twice a group: VGG-16-shaped fp32 262.8 -> 248.2 (100 % of the
+// copy rate), bf16 g 235.3 -> 219.0 (95 %), at 25 % sent 335 -> 325;
+// ResNet-50-shaped at 22 % sent 94.4 -> 84.7, with a bf16 g 89.8 -> 78.7;
+// LSTM-shaped 65.6 -> 65.1. Eight placers that each serve two compute warps
+// and poll: 268, 255, 359, 106, 102 and 69.
 //
 // Deadlock freedom. Take the lowest group m that is claimed but whose
 // aggregate is not published. Groups below m have published aggregates, so
@@ -43,9 +55,10 @@
 // which frees every entry and buffer space they hold. The CTA holding m waits
 // for nothing else: a compute warp never waits for buffer space (a segment
 // without room goes to its slot), the producer waits only for entries of
-// older groups of its own CTA and for its ring, and the ring's stages are
-// released by the compute warps as soon as they have read them. So m is
-// completed and the argument repeats; no wait depends on which CTAs are
+// older groups of its own CTA and for its ring, the ring's stages are
+// released by the compute warps as soon as they have read them, and the
+// aggregate warp never waits for a look-back. So m is published and the
+// argument repeats; no wait depends on which CTAs are
 // resident. Every wait is nevertheless bounded in time; one that runs out
 // latches kDevErrTimeout, and the CTA stops (after its bulk copies have
 // landed).
@@ -65,16 +78,22 @@ namespace efs {
 
 constexpr int kLbProducerWarp = kSWarps;       // 16
 constexpr int kLbScanWarp = kSWarps + 1;       // 17
-constexpr int kLbPlaceWarp = kSWarps + 2;      // 18: the first placer warp
-constexpr int kLbPlaceWarps = 12;  // with 8, placement bounds calls that send ~a quarter of a
-                                   // vector; 12 cost nothing on sparser ones
-constexpr int kLbThreads = 32 * (kSWarps + 2 + kLbPlaceWarps);  // 960
+constexpr int kLbAggWarp = kSWarps + 2;        // 18
+constexpr int kLbPlaceWarp = kSWarps + 3;      // 19: the first placer warp
+constexpr int kLbPlaceWarps = 12;  // with 8, calls that send a quarter of a vector take 6 % longer
+constexpr int kLbThreads = 32 * (kSWarps + 3 + kLbPlaceWarps);  // 992
 static_assert(kLbThreads <= 1024, "one CTA of at most 1024 threads");
 constexpr uint32_t kLbGroupTiles = 2;          // tiles per claimed group (the placement
                                                // assumes 2: 32 segments, one per lane)
 constexpr uint32_t kLbGroupSegs = kLbGroupTiles * kSWarps;
 constexpr uint32_t kLbClaimAhead = 2;          // groups claimed before the producer needs them
-constexpr uint32_t kLbEntries = 8;             // groups of a CTA in flight or pending
+// Groups of a CTA in flight or pending. More entries let streaming run ahead
+// of the look-back; in dense calls they also let it run ahead of the placers,
+// whose buffers then overflow into the slots. Measured with 8, 10, 12, 16 and 24, us a
+// call: VGG-16-shaped 262.0, 252.7, 248.2, 249.6, 252.0; with 5, 6, 7, 8 and 10 on the
+// shallow ring: ResNet-50-shaped at 22 % sent 82.2, 81.1, 84.7, 86.3, 87.0;
+// VGG-16-shaped at 25 % sent 365, 335, 325, 319, 322.
+constexpr int kLbManyEntries = 12, kLbFewEntries = 7;
 constexpr uint32_t kLbStageEnd = 0xffffffffu;
 constexpr uint32_t kLbSuspendNs = 1000;        // a suspended wait re-checks its flag and limit this often
 constexpr uint32_t kLbSegsPerLane = kLbGroupSegs / 32;  // segments per lane in the offset scan
@@ -82,27 +101,29 @@ static_assert(kLbGroupSegs % 32 == 0 && kLbSegsPerLane <= 2, "segments per look-
 
 // One group of a CTA, from the producer taking it until its pairs are placed.
 struct LbEntry {
-  uint32_t cnt[kLbGroupSegs];  // pairs of segment (q, w) at q * 16 + w
+  uint32_t seg[kLbGroupSegs];  // segment (q, w) at q * 16 + w: its pairs and where they are
   uint32_t off[kLbGroupSegs];  // output position of each segment's first pair
   FF err[kSWarps];             // the warps' shares of ||e'||^2 in this group
-  uint32_t tag;                // (claim number << 2) | state: 0 counting, 1 aggregate
-                               // published, 2 offsets ready
   uint32_t group;              // group index
-  uint32_t ntiles;             // tiles of the group (the last group may have fewer)
-  uint32_t arrivals;           // segments counted so far (complete: ntiles * 16)
-  uint32_t total;              // the group's aggregate (once complete)
-  uint32_t placed;             // kSWarps: the entry is free (set by the placers)
-  uint32_t spilled;            // bit l: segment l's pairs are in its global slot
+  uint32_t ntiles;             // tiles of the group (the last may have fewer); 0: no more groups
+  uint32_t placed;             // placers done with it
   uint32_t pad;
 };
-__device__ __forceinline__ uint32_t lb_tag(uint32_t seq, uint32_t state) { return (seq << 2) | state; }
+// A segment's word: its pairs (at most 256), whether they are in its global
+// slot, and else the position of the first in its warp's buffer.
+__device__ __forceinline__ uint32_t lb_seg(uint32_t count, bool slot, uint32_t first) {
+  return count | (slot ? 0x8000u : 0u) | (first << 16);
+}
+__device__ __forceinline__ uint32_t lb_seg_count(uint32_t seg) { return seg & 0x1ffu; }
+__device__ __forceinline__ bool lb_seg_slot(uint32_t seg) { return (seg & 0x8000u) != 0; }
+__device__ __forceinline__ uint32_t lb_seg_first(uint32_t seg) { return seg >> 16; }
 
-template <class Op, int kStages>
+template <class Op, int kStages, int kEntries>
 struct LbLayout {
   static constexpr uint32_t kRing = kStages * Op::kStageBytes;
   // pair buffer per compute warp: what is left of 227 KB (less 2 KB of static
   // shared memory), in whole warps of pairs
-  static constexpr uint32_t kEntryBytes = kLbEntries * sizeof(LbEntry);
+  static constexpr uint32_t kEntryBytes = kEntries * sizeof(LbEntry);
   static constexpr uint32_t kBudget = 227u * 1024u - 2048u;
   static constexpr uint32_t kFifo = ((kBudget - kRing - kEntryBytes) / (kSWarps * 8u)) / 32u * 32u;
   // (a segment that finds no room goes to its global slot, so nothing waits
@@ -118,8 +139,8 @@ struct LbArgs {
   double* err_out;      // optional: sum of a^2 over the coordinates whose residual is final
                         // here (not selected, not deferred), or null
   FF* err_parts;        // [groups] the groups' shares of it (used when err_out is set)
-  uint32_t* slot_idx;   // [num_tiles * 16 * 256] a segment's pairs when its warp's buffer is
-  float* slot_val;      // full: segment (tile, warp) at (tile * 16 + warp) * 256
+  uint2* slot;          // [num_tiles * 16 * 256] a segment's pairs (index, value bits) when its
+                        // warp's buffer is full: segment (tile, warp) at (tile * 16 + warp) * 256
   uint32_t* density_out;  // optional (host-mapped): the call's pair count * 65536 / d, a hint
                           // the host reads for later calls' choice of ring depth, or null
 };
@@ -166,16 +187,17 @@ __device__ __forceinline__ bool lb_mbar_wait(uint64_t* bar, uint32_t parity, uin
   }
 }
 
+// The barriers of an entry complete one phase per group that uses it.
+template <int kEntries>
+__device__ __forceinline__ uint32_t lb_parity(uint32_t seq) {
+  return (seq / kEntries) & 1u;
+}
+
 // x[j] for a run-time j without an indexed (local-memory) access.
 __device__ __forceinline__ float lb_pick(const float (&x)[4], int j) {
   const float lo = (j & 1) ? x[1] : x[0];
   const float hi = (j & 1) ? x[3] : x[2];
   return (j & 2) ? hi : lo;
-}
-
-// Named barrier of the placer warps (id 2; 0 is __syncthreads, 1 group_bar).
-__device__ __forceinline__ void lb_place_bar(int count) {
-  asm volatile("bar.sync 2, %0;" ::"r"(count) : "memory");
 }
 
 // The test hook withholds a tile; here the group holding it never publishes.
@@ -184,7 +206,7 @@ __device__ __forceinline__ bool lb_withheld(const ScanCtx& ctx, uint32_t group) 
          static_cast<int64_t>(group) == ctx.withheld_tile / static_cast<int64_t>(kLbGroupTiles);
 }
 
-template <class Op, int kStages>
+template <class Op, int kStages, int kEntries>
 __global__ void __launch_bounds__(kLbThreads, 1)
     lookback_stream_kernel(Op op, uint32_t* __restrict__ idx_out,
                            float* __restrict__ val_out, uint32_t* __restrict__ count_out,
@@ -193,20 +215,19 @@ __global__ void __launch_bounds__(kLbThreads, 1)
   __shared__ __align__(8) uint64_t s_full[kStages];
   __shared__ __align__(8) uint64_t s_empty[kStages];
   __shared__ uint32_t s_stage_tile[kStages];  // tile of the stage's current use, or the end
-  __shared__ uint32_t s_stage_info[kStages];  // its group's entry slot | (tile in the group << 8)
-  __shared__ uint32_t s_claimed;              // groups the producer took so far
-  __shared__ uint32_t s_claim_done;           // the producer takes no more
+  __shared__ uint32_t s_stage_slot[kStages];  // its group's entry
+  __shared__ __align__(8) uint64_t s_counted[kEntries];  // every segment's word is there
+  __shared__ __align__(8) uint64_t s_ready[kEntries];    // so are the output positions
+  __shared__ __align__(8) uint64_t s_free[kEntries];     // every pair is placed, the total published
   __shared__ uint32_t s_failed;               // a wait of this CTA ran out
   __shared__ uint32_t s_resolved;             // groups the look-back warp resolved
   __shared__ uint32_t s_freed[kSWarps];       // pairs of each compute warp placed so far
-  __shared__ uint32_t s_place_go;             // the placers' next group is ready (else: stop)
   __shared__ uint32_t s_cq[kLbClaimAhead];    // groups claimed ahead, with the queue counts
   __shared__ uint32_t s_cq_tail, s_cq_head;
   __shared__ uint32_t s_last;                 // this CTA finished last
   __shared__ FF s_err_sum[32];
-  using L = LbLayout<Op, kStages>;
-  uint32_t* const f_idx = reinterpret_cast<uint32_t*>(smem + L::kRing);
-  float* const f_val = reinterpret_cast<float*>(smem + L::kRing + kSWarps * L::kFifo * 4u);
+  using L = LbLayout<Op, kStages, kEntries>;
+  uint2* const f_pair = reinterpret_cast<uint2*>(smem + L::kRing);  // (index, value bits)
   LbEntry* const ent = reinterpret_cast<LbEntry*>(smem + L::kOffEntries);
 
   const uint32_t T = ctx.num_tiles;
@@ -218,19 +239,18 @@ __global__ void __launch_bounds__(kLbThreads, 1)
       mbar_init(&s_full[s], 1);
       mbar_init(&s_empty[s], kSWarps);
     }
+    for (uint32_t s = 0; s < kEntries; ++s) {
+      mbar_init(&s_counted[s], kSWarps);
+      mbar_init(&s_ready[s], 1);
+      mbar_init(&s_free[s], 2);  // the aggregate warp and the last placer
+    }
     mbar_init_fence();
-    s_claimed = 0;
-    s_claim_done = 0;
     s_failed = 0;
     s_resolved = 0;
     s_cq_tail = 0;
     s_cq_head = 0;
   }
   if (threadIdx.x < kSWarps) s_freed[threadIdx.x] = 0;
-  if (threadIdx.x < kLbEntries) {
-    ent[threadIdx.x].placed = kSWarps;  // free
-    ent[threadIdx.x].tag = 0xffffffffu;
-  }
   __syncthreads();
   // A dependent launch starts while the previous kernel's last groups are
   // placed, a phase that leaves DRAM mostly idle: pull the first groups the
@@ -279,9 +299,10 @@ __global__ void __launch_bounds__(kLbThreads, 1)
       };
       uint32_t cq_head = 0;
       while (ok) {
-        const uint32_t slot = seq % kLbEntries;
+        const uint32_t slot = seq % kEntries;
         LbEntry& en = ent[slot];
-        if (!lb_spin([&] { return vld(en.placed) == kSWarps; }, &s_failed, ctx)) {
+        if (seq >= kEntries &&
+            !lb_mbar_wait(&s_free[slot], lb_parity<kEntries>(seq) ^ 1u, &s_failed, ctx)) {
           ok = false;
           break;
         }
@@ -292,41 +313,29 @@ __global__ void __launch_bounds__(kLbThreads, 1)
         __threadfence_block();  // the claimed number after the count
         const uint32_t g = vld(s_cq[cq_head % kLbClaimAhead]);
         vst(s_cq_head, ++cq_head);
-        if (g >= G) break;
-        const uint32_t nt = min(kLbGroupTiles, T - g * kLbGroupTiles);
+        const uint32_t nt = g < G ? min(kLbGroupTiles, T - g * kLbGroupTiles) : 0u;
         en.group = g;
         en.ntiles = nt;
-        en.arrivals = 0;
-        en.spilled = 0;
         en.placed = 0;
-        __threadfence_block();
-        vst(en.tag, lb_tag(seq, 0));
-        vst(s_claimed, seq + 1);
-        for (uint32_t q = 0; q < nt; ++q, ++r) {
+        // the group's stages; none left: one that ends the compute warps, whose
+        // arrivals carry the entry's end mark (ntiles == 0) to the other roles
+        for (uint32_t q = 0; q < (nt ? nt : 1u); ++q, ++r) {
           const int s = static_cast<int>(r % kStages);
           if (!stage_free(s)) {
             ok = false;
             break;
           }
           const uint32_t t = g * kLbGroupTiles + q;
-          s_stage_tile[s] = t;
-          s_stage_info[s] = slot | (q << 8);
-          if (op.full(t))
+          s_stage_tile[s] = nt ? t : kLbStageEnd;
+          s_stage_slot[s] = slot;
+          if (nt && op.full(t))
             op.fill(smem + s * Op::kStageBytes, t, &s_full[s], policy);
           else
             mbar_arrive(&s_full[s]);  // a partial tile is read from global memory
         }
         ++seq;
+        if (!nt) break;
       }
-      if (ok) {  // the end marker
-        const int s = static_cast<int>(r % kStages);
-        if (stage_free(s)) {
-          s_stage_tile[s] = kLbStageEnd;
-          mbar_arrive(&s_full[s]);
-          ++r;
-        }
-      }
-      vst(s_claim_done, 1u);
       griddep_launch_dependents();  // this CTA reads nothing more: the next kernel may be scheduled
       // no copy may land after the CTA exits: wait for the last use of every
       // stage (a completed phase reports complete at once)
@@ -337,20 +346,32 @@ __global__ void __launch_bounds__(kLbThreads, 1)
   } else if (warp == kLbScanWarp) {
     // ------------------------------------------------------ look-back
     for (uint32_t seq = 0;; ++seq) {
-      uint32_t go = 0;
-      if (lane == 0) {
-        lb_spin([&] { return vld(s_claimed) > seq || vld(s_claim_done) != 0; }, &s_failed, ctx);
-        go = vld(s_claimed) > seq && !vld(s_failed);
-        if (go) {
-          LbEntry& en = ent[seq % kLbEntries];
-          go = lb_spin([&] { return vld(en.tag) == lb_tag(seq, 1); }, &s_failed, ctx);
-        }
-        __threadfence_block();
+      const uint32_t slot = seq % kEntries;
+      LbEntry& en = ent[slot];
+      const bool counted = lb_mbar_wait(&s_counted[slot], lb_parity<kEntries>(seq), &s_failed, ctx);
+      if (!__all_sync(0xffffffffu, counted)) break;
+      const uint32_t g = en.group, nt = en.ntiles;
+      if (nt == 0) {  // no more groups: the placers end too
+        if (lane == 0) mbar_arrive(&s_ready[slot]);
+        break;
       }
-      if (!__shfl_sync(0xffffffffu, go, 0)) break;
-      __syncwarp();
-      LbEntry& en = ent[seq % kLbEntries];
-      const uint32_t g = en.group, nt = en.ntiles, total = en.total;
+      // segment positions in (tile, warp) order: lane l holds segments
+      // l * kLbSegsPerLane onwards
+      const uint32_t nseg = nt * kSWarps;
+      uint32_t cs[kLbSegsPerLane], mine = 0;
+#pragma unroll
+      for (uint32_t i = 0; i < kLbSegsPerLane; ++i) {
+        const uint32_t sg = lane * kLbSegsPerLane + i;
+        cs[i] = sg < nseg ? lb_seg_count(en.seg[sg]) : 0u;
+        mine += cs[i];
+      }
+      uint32_t incl = mine;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t v = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += v;
+      }
+      const uint32_t total = __shfl_sync(0xffffffffu, incl, 31);
       bool timed_out = false;
       const uint32_t excl = lookback_exclusive(ctx, g, timed_out);
       if (timed_out) {
@@ -362,22 +383,6 @@ __global__ void __launch_bounds__(kLbThreads, 1)
       }
       if (lane == 0 && !lb_withheld(ctx, g))
         st_relaxed_u64(ctx.status + g, pack_status(ctx.epoch, kFlagPrefix, excl + total));
-      // segment positions in (tile, warp) order: lane l holds segments
-      // l * kLbSegsPerLane onwards
-      const uint32_t nseg = nt * kSWarps;
-      uint32_t cs[kLbSegsPerLane], mine = 0;
-#pragma unroll
-      for (uint32_t i = 0; i < kLbSegsPerLane; ++i) {
-        const uint32_t sg = lane * kLbSegsPerLane + i;
-        cs[i] = sg < nseg ? en.cnt[sg] : 0u;
-        mine += cs[i];
-      }
-      uint32_t incl = mine;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t v = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += v;
-      }
       const uint32_t first = excl + incl - mine;
       uint32_t run = first;
 #pragma unroll
@@ -407,114 +412,110 @@ __global__ void __launch_bounds__(kLbThreads, 1)
       }
       __syncwarp();
       if (lane == 0) {
-        __threadfence_block();
-        vst(en.tag, lb_tag(seq, 2));
+        mbar_arrive(&s_ready[slot]);
         ++s_resolved;
+      }
+    }
+  } else if (warp == kLbAggWarp) {
+    // ------------------------------------------------------ aggregates
+    // Publishes each group's total as soon as its segments are counted (the
+    // look-back warp may still be waiting for an earlier group's neighbours).
+    for (uint32_t seq = 0;; ++seq) {
+      const uint32_t slot = seq % kEntries;
+      const bool counted = lb_mbar_wait(&s_counted[slot], lb_parity<kEntries>(seq), &s_failed, ctx);
+      if (!__all_sync(0xffffffffu, counted)) break;
+      const LbEntry& en = ent[slot];
+      const uint32_t g = en.group, nseg = en.ntiles * kSWarps;
+      if (nseg == 0) break;
+      uint32_t part = 0;
+#pragma unroll
+      for (uint32_t i = 0; i < kLbSegsPerLane; ++i) {
+        const uint32_t sg = lane + 32 * i;
+        part += sg < nseg ? lb_seg_count(en.seg[sg]) : 0u;
+      }
+      const uint32_t agg = warp_sum(part);
+      if (lane == 0) {
+        // max: the look-back warp may have published the group's prefix, whose
+        // flag is the larger one
+        if (!lb_withheld(ctx, g))
+          atomicMax(reinterpret_cast<unsigned long long*>(ctx.status + g),
+                    static_cast<unsigned long long>(pack_status(ctx.epoch, kFlagAggregate, agg)));
+        mbar_arrive(&s_free[slot]);  // done with the entry
       }
     }
   } else if (warp >= kLbPlaceWarp) {
     // ------------------------------------------------------ placement
-    // For each group in claim order, once its offsets are there: its pairs,
-    // in (tile, warp) order, are the output positions [off[0], off[0] + n).
-    // The kLbPlaceWarps warps copy them together, lane k of placer warp p
-    // taking the positions = 32 p + k modulo 32 kLbPlaceWarps, each from its
-    // compute warp's buffer (coalesced stores); then the buffers' space is
-    // handed back and the entry freed. Every placer warp tracks the buffer
-    // heads itself (lane w < 16: compute warp w's oldest unplaced pair).
+    // For each group in claim order, once its positions are there: placer p
+    // copies the segments l = p, p + kLbPlaceWarps, ...: a segment's pairs are
+    // consecutive in its source and in the output, so the warp's lanes take
+    // consecutive pairs (coalesced loads and stores). No placer waits for
+    // another. The last to finish a group hands the buffers' space back and
+    // frees the entry: every placer goes through the groups in order, so all
+    // earlier groups' pairs are placed by then.
     const int pw = warp - kLbPlaceWarp;
-    constexpr int kPlaceThreads = 32 * kLbPlaceWarps;
     const uint64_t keep_policy = Op::kKeepPairs ? l2_evict_last_policy() : 0ull;
-    uint32_t head = 0;
     bool overflow = false;
     for (uint32_t seq = 0;; ++seq) {
-      if (pw == 0 && lane == 0) {
-        lb_spin([&] { return vld(s_claimed) > seq || vld(s_claim_done) != 0; }, &s_failed, ctx);
-        uint32_t go = vld(s_claimed) > seq && !vld(s_failed);
-        if (go) {
-          LbEntry& en = ent[seq % kLbEntries];
-          go = lb_spin([&] { return vld(en.tag) == lb_tag(seq, 2); }, &s_failed, ctx);
-        }
-        s_place_go = go;
-      }
-      lb_place_bar(kPlaceThreads);  // the decision and the offsets are visible to every placer
-      if (!s_place_go) break;
-      LbEntry& en = ent[seq % kLbEntries];
-      const uint32_t nseg = en.ntiles * kSWarps;
-      // lane l describes segment l (l < nseg): start within the group, count,
-      // and its first pair's buffer position
-      const uint32_t c = static_cast<uint32_t>(lane) < nseg ? en.cnt[lane] : 0u;
-      const uint32_t first = en.off[0];
-      const uint32_t start = static_cast<uint32_t>(lane) < nseg ? en.off[lane] - first : 0xffffffffu;
-      const uint32_t spilled = en.spilled;
-      const bool in_slot = (spilled >> lane) & 1u;
-      const uint32_t c_buf = in_slot ? 0u : c;  // pairs the segment holds in its warp's buffer
-      const int w = lane & (kSWarps - 1);
-      // a buffered segment's first pair: its warp's head, after the warp's
-      // tile-0 segment when that one is buffered too (kLbGroupTiles == 2); a
-      // slotted segment's: its slot's number
-      uint32_t src = __shfl_sync(0xffffffffu, head, w);
-      const uint32_t c_prev = __shfl_sync(0xffffffffu, c_buf, (lane - kSWarps) & 31);
-      if (lane >= kSWarps) src += c_prev;
-      if (src >= L::kFifo) src -= L::kFifo;
-      if (in_slot)
-        src = (en.group * kLbGroupTiles + static_cast<uint32_t>(lane) / kSWarps) * kSWarps +
-              static_cast<uint32_t>(w);
-      // placer warp p copies the segments l = p, p + kLbPlaceWarps, ...: the
-      // segment's pairs are consecutive in its source and in the output, so
-      // the warp's lanes take consecutive pairs (coalesced loads and stores)
+      const uint32_t slot = seq % kEntries;
+      LbEntry& en = ent[slot];
+      const bool ready = lb_mbar_wait(&s_ready[slot], lb_parity<kEntries>(seq), &s_failed, ctx);
+      if (!__all_sync(0xffffffffu, ready)) break;
+      const uint32_t nt = en.ntiles;
+      if (nt == 0) break;
+      const uint32_t nseg = nt * kSWarps;
+      // lane l describes segment l (l < nseg)
+      const uint32_t seg = static_cast<uint32_t>(lane) < nseg ? en.seg[lane] : 0u;
+      const uint32_t dst = en.off[lane];
       for (int l = pw; l < static_cast<int>(nseg); l += kLbPlaceWarps) {
-        const uint32_t cl = __shfl_sync(0xffffffffu, c, l);
-        const uint32_t dl = first + __shfl_sync(0xffffffffu, start, l);
-        const uint32_t sl = __shfl_sync(0xffffffffu, src, l);
-        const bool slotted = (spilled >> l) & 1u;
+        const uint32_t sl = __shfl_sync(0xffffffffu, seg, l);
+        const uint32_t dl = __shfl_sync(0xffffffffu, dst, l);
+        const uint32_t cl = lb_seg_count(sl), first = lb_seg_first(sl);
+        const bool slotted = lb_seg_slot(sl);
         const uint32_t fbase = static_cast<uint32_t>(l & (kSWarps - 1)) * L::kFifo;
+        const size_t sbase =
+            (static_cast<size_t>(en.group * kLbGroupTiles) * kSWarps + l) * kSWarpElems;
         for (uint32_t k = lane; k < cl; k += 32) {
-          uint32_t xi;
-          float xv;
+          uint2 x;
           if (slotted) {
-            const size_t b = static_cast<size_t>(sl) * kSWarpElems + k;
-            xi = la.slot_idx[b];  // written by a warp of this CTA (ordered by the fences)
-            xv = la.slot_val[b];
+            x = la.slot[sbase + k];  // written by a warp of this CTA (ordered by the barriers)
           } else {
-            uint32_t b = sl + k;
+            uint32_t b = first + k;
             if (b >= L::kFifo) b -= L::kFifo;
-            xi = f_idx[fbase + b];
-            xv = f_val[fbase + b];
+            x = f_pair[fbase + b];
           }
           const uint32_t pos = dl + k;
           if (pos < cap) {
             if constexpr (Op::kKeepPairs) {
-              st_pair_policy(idx_out + pos, val_out + pos, xi, xv, keep_policy);
+              st_pair_policy(idx_out + pos, val_out + pos, x.x, __uint_as_float(x.y), keep_policy);
             } else {
-              idx_out[pos] = xi;
-              val_out[pos] = xv;
+              idx_out[pos] = x.x;
+              val_out[pos] = __uint_as_float(x.y);
             }
           } else {
             overflow = true;
           }
         }
       }
-      // every compute warp's buffer head moves past its pairs of the group
-      const uint32_t c_tile1 = __shfl_sync(0xffffffffu, c_buf, (lane + kSWarps) & 31);
-      const uint32_t mine_total = c_buf + (lane < kSWarps ? c_tile1 : 0u);
-      if (lane < kSWarps) {
-        head += mine_total;
-        if (head >= L::kFifo) head -= L::kFifo;
+      __syncwarp();  // every lane has read its pairs and the entry
+      uint32_t before = 0;
+      if (lane == 0) {
+        __threadfence_block();
+        before = atomicAdd(&en.placed, 1u);
       }
-      lb_place_bar(kPlaceThreads);  // every placer is done with the buffers and the entry
-      if (pw == 0) {
-        if (lane < kSWarps) atomicAdd(&s_freed[lane], mine_total);
-        if (lane == 0) {
-          __threadfence_block();
-          vst(en.placed, kSWarps);  // the entry is free
-        }
+      before = __shfl_sync(0xffffffffu, before, 0);
+      if (before == kLbPlaceWarps - 1) {
+        __threadfence_block();  // the other placers' reads, before the space is handed back
+        const uint32_t in_buffer = lb_seg_slot(seg) ? 0u : lb_seg_count(seg);
+        const uint32_t both = in_buffer + __shfl_down_sync(0xffffffffu, in_buffer, kSWarps);
+        if (lane < kSWarps) atomicAdd(&s_freed[lane], both);
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&s_free[slot]);
       }
     }
     if (__any_sync(0xffffffffu, overflow) && lane == 0) atomicOr(ctx.error, kDevErrOverflow);
   } else {
     // ------------------------------------------------------ compute warps
-    uint32_t* const my_idx = f_idx + warp * L::kFifo;
-    float* const my_val = f_val + warp * L::kFifo;
+    uint2* const my_pair = f_pair + warp * L::kFifo;
     uint32_t tail = 0;      // next buffer position this warp writes
     uint32_t appended = 0;  // pairs appended so far (the placer counts the freed ones)
     FF warp_err{0.0f, 0.0f};  // lane 0: share of ||e'||^2 in the current group
@@ -549,8 +550,11 @@ __global__ void __launch_bounds__(kLbThreads, 1)
       bool arrived = lb_mbar_wait(&s_full[s], (r / kStages) & 1u, &s_failed, ctx);
       if (!__all_sync(0xffffffffu, arrived)) break;
       const uint32_t t0 = s_stage_tile[s];
-      const uint32_t slot = s_stage_info[s] & 0xffu;
-      if (t0 == kLbStageEnd) break;
+      const uint32_t slot = s_stage_slot[s];
+      if (t0 == kLbStageEnd) {
+        if (lane == 0) mbar_arrive(&s_counted[slot]);  // the end mark, for the other roles
+        break;
+      }
       LbEntry& en = ent[slot];
       const uint32_t nt = en.ntiles;
       float a[kLbGroupTiles][kSUnits][4];
@@ -613,8 +617,8 @@ __global__ void __launch_bounds__(kLbThreads, 1)
             uint32_t p = off[q][v];
             for (uint32_t bits = sel[q][v] & 0xfu; bits; bits &= bits - 1, ++p) {
               const int j = __ffs(bits) - 1;
-              la.slot_idx[sb + p] = first_elem + v * 128 + j;
-              la.slot_val[sb + p] = lb_pick(a[q][v], j);
+              la.slot[sb + p] =
+                  make_uint2(first_elem + v * 128 + j, __float_as_uint(lb_pick(a[q][v], j)));
             }
           }
         } else {
@@ -624,50 +628,28 @@ __global__ void __launch_bounds__(kLbThreads, 1)
             if (p >= L::kFifo) p -= L::kFifo;
             for (uint32_t bits = sel[q][v] & 0xfu; bits; bits &= bits - 1) {
               const int j = __ffs(bits) - 1;
-              my_idx[p] = first_elem + v * 128 + j;
-              my_val[p] = lb_pick(a[q][v], j);
+              my_pair[p] =
+                  make_uint2(first_elem + v * 128 + j, __float_as_uint(lb_pick(a[q][v], j)));
               if (++p == L::kFifo) p = 0;
             }
           }
         }
       }
-      tail += buf_total;
-      if (tail >= L::kFifo) tail -= L::kFifo;
-      appended += buf_total;
-      uint32_t before = 0;
+      __syncwarp();  // every lane's pairs before the arrival
       if (lane == 0) {
-        en.cnt[warp] = seg_total[0];
-        if (nt == 2) en.cnt[kSWarps + warp] = seg_total[1];
-        if (to_slot)
-          atomicOr(&en.spilled, ((to_slot & 1u) << warp) | ((to_slot >> 1) << (kSWarps + warp)));
+        en.seg[warp] = lb_seg(seg_total[0], to_slot & 1u, tail);
+        uint32_t first1 = tail + ((to_slot & 1u) ? 0u : seg_total[0]);
+        if (first1 >= L::kFifo) first1 -= L::kFifo;
+        if (nt == 2) en.seg[kSWarps + warp] = lb_seg(seg_total[1], to_slot & 2u, first1);
         if (la.err_out) {
           en.err[warp] = warp_err;
           warp_err = FF{0.0f, 0.0f};
         }
-        __threadfence_block();  // the pairs and the counts before the arrival
-        before = atomicAdd(&en.arrivals, nt);
+        mbar_arrive(&s_counted[slot]);  // releases the pairs and the words
       }
-      before = __shfl_sync(0xffffffffu, before, 0);
-      if (before + nt == nt * kSWarps) {
-        // this warp counted the group's last segments: its aggregate
-        if (lane == 0) __threadfence_block();
-        __syncwarp();
-        const uint32_t nseg = nt * kSWarps;
-        uint32_t part = 0;
-#pragma unroll
-        for (uint32_t i = 0; i < kLbSegsPerLane; ++i) {
-          const uint32_t sg = lane + 32 * i;
-          part += sg < nseg ? vld(en.cnt[sg]) : 0u;
-        }
-        const uint32_t agg = warp_sum(part);
-        if (lane == 0) {
-          if (!lb_withheld(ctx, en.group))
-            st_relaxed_u64(ctx.status + en.group, pack_status(ctx.epoch, kFlagAggregate, agg));
-          en.total = agg;
-          __threadfence_block();
-          vst(en.tag, vld(en.tag) | 1u);  // (claim number, 0) -> (claim number, 1)
-        }
-      }
+      tail += buf_total;
+      if (tail >= L::kFifo) tail -= L::kFifo;
+      appended += buf_total;
     }
   }
 

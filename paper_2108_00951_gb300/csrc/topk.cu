@@ -300,6 +300,14 @@ struct TopkCandOp : StreamIn<GT, kAny> {
 };
 
 constexpr int kTkStages = 4;
+// the claimed-group kernel of the candidate pass
+template <typename GT, bool kAny>
+using GroupLayout = LbLayout<TopkCandOp<GT, kAny>, kTkStages, kLbManyEntries>;
+template <typename GT, bool kAny>
+const void* group_kernel() {
+  return reinterpret_cast<const void*>(
+      &lookback_stream_kernel<TopkCandOp<GT, kAny>, kTkStages, kLbManyEntries>);
+}
 
 // The candidate bound of the streaming pass, in a kernel of its own before
 // it: every CTA histograms the top 13 key bits of 2048 coordinates spread
@@ -1044,9 +1052,8 @@ __global__ void __launch_bounds__(kSelThreads, 1)
 
 template <typename GT, bool kAny>
 int tk_group_blocks_per_sm() {
-  const void* fn =
-      reinterpret_cast<const void*>(&lookback_stream_kernel<TopkCandOp<GT, kAny>, kTkStages>);
-  const uint32_t smem = LbLayout<TopkCandOp<GT, kAny>, kTkStages>::kSmem;
+  const void* fn = group_kernel<GT, kAny>();
+  const uint32_t smem = GroupLayout<GT, kAny>::kSmem;
   int n = 0;
   if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fn, kLbThreads, smem) != cudaSuccess)
@@ -1131,11 +1138,10 @@ cudaError_t launch_typed(const GT* g, float* e, float gamma, uint32_t k, uint32_
     const uint32_t gslots = static_cast<uint32_t>(per_sm_groups * dev.sm_count);
     const uint32_t ggrid = groups < gslots ? groups : gslots;
     LbArgs la{nullptr, err_out ? ws.stream_err() : nullptr, reinterpret_cast<FF*>(ws.counts()),
-              ws.stage_idx(), ws.stage_val()};
+              ws.stage_pairs()};
     void* gp[] = {&op, &args.list_idx, &args.list_val, &args.list_count, &cap, &ctx, &la};
-    err = launch_pdl(
-        reinterpret_cast<const void*>(&lookback_stream_kernel<TopkCandOp<GT, kAny>, kTkStages>), ggrid,
-        kLbThreads, LbLayout<TopkCandOp<GT, kAny>, kTkStages>::kSmem, ws.stream, gp, false);
+    err = launch_pdl(group_kernel<GT, kAny>(), ggrid, kLbThreads, GroupLayout<GT, kAny>::kSmem,
+                     ws.stream, gp, false);
   } else {
     StreamArgs sa{ws.stage_idx(), ws.stage_val(), ws.counts(), ws.chunks(), nullptr,
                   err_out ? ws.stream_err() : nullptr, ws.errparts()};

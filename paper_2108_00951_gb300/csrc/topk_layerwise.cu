@@ -309,6 +309,15 @@ struct LwCandOp : StreamIn<GT, kAny> {
   }
 };
 
+// the claimed-group kernel of the candidate pass
+template <typename GT, bool kAny>
+using GroupLayout = LbLayout<LwCandOp<GT, kAny>, kLwStages, kLbManyEntries>;
+template <typename GT, bool kAny>
+const void* group_kernel() {
+  return reinterpret_cast<const void*>(
+      &lookback_stream_kernel<LwCandOp<GT, kAny>, kLwStages, kLbManyEntries>);
+}
+
 // ------------------------------------------------------------- 3 select
 struct LwArgs {
   const LwSeg* segs;
@@ -789,8 +798,8 @@ __global__ void __launch_bounds__(kLwThreads, 1)
 // ------------------------------------------------------------- host side
 template <typename GT, bool kAny>
 int lw_group_blocks_per_sm() {
-  const void* fn = reinterpret_cast<const void*>(&lookback_stream_kernel<LwCandOp<GT, kAny>, kLwStages>);
-  const uint32_t smem = LbLayout<LwCandOp<GT, kAny>, kLwStages>::kSmem;
+  const void* fn = group_kernel<GT, kAny>();
+  const uint32_t smem = GroupLayout<GT, kAny>::kSmem;
   int n = 0;
   if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fn, kLbThreads, smem) != cudaSuccess)
@@ -874,11 +883,10 @@ cudaError_t launch_typed(const GT* g, float* e, float gamma, uint32_t d, uint32_
     const uint32_t gslots = static_cast<uint32_t>(per_sm_groups * dev.sm_count);
     const uint32_t ggrid = groups < gslots ? groups : gslots;
     LbArgs la{tile_base, err_out ? ws.stream_err() : nullptr, reinterpret_cast<FF*>(ws.counts()),
-              ws.stage_idx(), ws.stage_val()};
+              ws.stage_pairs()};
     void* gp[] = {&op, &list_idx, &list_val, &list_count, &cap, &ctx, &la};
-    err = launch_pdl(
-        reinterpret_cast<const void*>(&lookback_stream_kernel<LwCandOp<GT, kAny>, kLwStages>), ggrid,
-        kLbThreads, LbLayout<LwCandOp<GT, kAny>, kLwStages>::kSmem, ws.stream, gp, false);
+    err = launch_pdl(group_kernel<GT, kAny>(), ggrid, kLbThreads, GroupLayout<GT, kAny>::kSmem,
+                     ws.stream, gp, false);
   } else {
     StreamArgs sa{ws.stage_idx(), ws.stage_val(), ws.counts(), ws.chunks(), tile_base,
                   err_out ? ws.stream_err() : nullptr, ws.errparts()};
