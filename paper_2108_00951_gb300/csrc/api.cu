@@ -559,7 +559,7 @@ ef_status int_aggregate(uint32_t n, const int32_t* const* q, uint64_t d, int32_t
   st = acquire_workspace(s, 0, 0, 0, 0, &ws);
   if (st != EF_OK) return st;
   return finish_launch(
-      launch_int_aggregate(n, q, static_cast<uint32_t>(d), scale_log2, dense_out, *ws, info), ws);
+      launch_int_aggregate(n, q, static_cast<uint32_t>(d), scale_log2, dense_out, *ws), ws);
 }
 
 ef_status ef_check_status(ef_stream_t stream) {

@@ -19,6 +19,7 @@ constexpr size_t kOffTileClaim = 24;    // uint32[3]: work dispenser: handed out
                                         // groups resolved (zero between calls)
 constexpr size_t kOffTkListCount = 72;  // uint32: candidates emitted by the streaming pass
 constexpr size_t kOffErrArrive = 80;    // uint32: arrivals of the e' norm pass (zero after it)
+constexpr size_t kOffRoundTotal = 84;   // uint32: coordinates the rounding did not send (zero after it)
 constexpr size_t kOffStreamErr = 88;    // double: the streaming pass's share of ||e'||^2
 // Per-call Top-k state that must start at zero, in two blocks used by
 // alternate calls on a workspace: a call's candidate stream zeroes the
@@ -232,7 +233,7 @@ cudaError_t launch_scaled_round(const void* g, bool g_bf16, float* e, float gamm
                                 uint32_t d, int32_t* q, uint32_t* unsent, double* err_out,
                                 Workspace& ws, const DeviceInfo& dev);
 cudaError_t launch_int_aggregate(uint32_t n, const int32_t* const* q, uint32_t d, int m,
-                                 float* dense_out, Workspace& ws, const DeviceInfo& dev);
+                                 float* dense_out, Workspace& ws);
 
 // Launch bookkeeping.
 // A launch that may begin while the previous kernel on the stream finishes
