@@ -462,10 +462,11 @@ void ef_test_set_lookback_fault(int64_t withheld_tile, uint32_t spin_limit_us);
  * below; for the hard-threshold step, a shallower ring with larger pair
  * buffers once an earlier call on the same stream sent at least 1/12 of its
  * coordinates), 1 static chunks, 2 claimed groups, 3 claimed groups with the
- * shallower ring (hard-threshold; the candidate passes treat 3 as 2). Any
- * other value means 0. The results are the same whichever kernel runs; the
- * hook lets tests run each on small inputs. Process-wide; never needed in
- * production.
+ * shallower ring (hard-threshold; the candidate passes treat 3 as 2). With 0, a
+ * Top-k call of at most 65,536 coordinates streams nothing: one thread-block
+ * cluster does all of it. Any other value means 0. The results are the same
+ * whichever kernel runs; the hook lets tests run each on small inputs.
+ * Process-wide; never needed in production.
  */
 void ef_test_set_stream_kernel(int mode);
 

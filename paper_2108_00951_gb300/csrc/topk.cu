@@ -37,6 +37,8 @@
 // full-array path adds a read of a per digit level and two for the output.
 #include <algorithm>
 
+#include <cooperative_groups.h>
+
 #include "internal.h"
 #include "select.cuh"
 #include "stream_lookback.cuh"
@@ -1050,6 +1052,215 @@ __global__ void __launch_bounds__(kSelThreads, 1)
   if (__syncthreads_or(overflow) && threadIdx.x == 0) atomicOr(args.error, kDevErrOverflow);
 }
 
+// --------------------------------------------------- short vectors, one launch
+// A vector that the shared memory of one thread-block cluster holds: every CTA
+// keeps its slice of a on chip, so g and e are read once and e written once,
+// with no candidate list and nothing left between launches. Three digit levels
+// of the magnitude bits (11, 10 and 10) narrow the threshold: each CTA
+// histograms the magnitudes that match the prefix, adds its bins to rank 0's
+// through distributed shared memory, and after a cluster barrier reads the
+// merged bins and picks the same one; equal magnitudes at the last level go in
+// position order. One more barrier exchanges the slices' counts; the slices
+// are then written in order.
+// What it saves is launches and the waits between them; what it costs is the
+// rate of 8 SMs instead of 152. Measured on a GB300, us a call from Python,
+// three launches -> one: d = 500 16.7 -> 11.4, 20,000 18.0 -> 13.9, 45,000
+// 17.8 -> 15.1 (k = 0.2 %) and 22.4 -> 16.5 (10 %), 65,000 17.7 -> 16.2 and
+// 22.8 -> 18.0, but 100,000 18.5 -> 22.3. With clusters of 16: 14.3 at 500,
+// 17.4 at 45,000, 18.2 at 65,000.
+constexpr int kClusterCtas = 8;             // the portable cluster size
+constexpr uint32_t kClusterSlice = 8192;    // values of a slice in shared memory
+constexpr uint32_t kClusterMax = kClusterCtas * kClusterSlice;
+constexpr uint32_t kClusterSmem = kClusterSlice * sizeof(float);
+
+template <typename GT>
+__global__ void __launch_bounds__(kSelThreads, 1)
+    topk_cluster_kernel(const GT* __restrict__ g, float* __restrict__ e, float gamma, uint32_t k,
+                        uint32_t d, uint32_t* __restrict__ idx_out, float* __restrict__ val_out,
+                        uint32_t* __restrict__ count_out, double* err_out) {
+  extern __shared__ __align__(16) float s_a[];
+  __shared__ uint32_t s_hist[kHistBins];
+  __shared__ uint32_t s_merged[3][kHistBins];  // rank 0's: the cluster's bins of a level
+  __shared__ uint32_t s_w[kSelThreads / 32];
+  __shared__ uint32_t s_above, s_equal;        // this slice's counts, read by the others
+  __shared__ FF s_share, s_ff[32];
+  namespace cg = cooperative_groups;
+  const cg::cluster_group cluster = cg::this_cluster();
+  const uint32_t rank = cluster.block_rank(), C = cluster.num_blocks();
+  const uint32_t tid = threadIdx.x;
+  const uint32_t per = ((d + C - 1) / C + 3u) & ~3u;
+  const uint32_t lo = min(rank * per, d), m = min(per, d - lo);
+  for (uint32_t b = tid; b < static_cast<uint32_t>(kHistBins); b += kSelThreads) {
+    s_hist[b] = 0;
+    for (int l = 0; l < 3; ++l) s_merged[l][b] = 0;
+  }
+  __syncthreads();
+  griddep_wait();  // g and e may come from the kernels before
+  griddep_launch_dependents();
+  constexpr int kBatch = 8;  // loads of g and of e in flight per thread
+  const uint32_t lane = tid & 31;
+  for (uint32_t w0 = tid & ~31u; w0 < m; w0 += kBatch * kSelThreads) {  // whole warps
+    float gv[kBatch], ev[kBatch];
+#pragma unroll
+    for (int j = 0; j < kBatch; ++j) {
+      const uint32_t i = w0 + lane + j * kSelThreads;
+      gv[j] = i < m ? grad_scalar(g, lo + i) : 0.0f;
+      ev[j] = i < m ? e[lo + i] : 0.0f;
+    }
+#pragma unroll
+    for (int j = 0; j < kBatch; ++j) {
+      const uint32_t i = w0 + lane + j * kSelThreads;
+      const float a = __fmaf_rn(gamma, gv[j], ev[j]);
+      const uint32_t bin = (__float_as_uint(a) & 0x7fffffffu) >> 20;
+      if (i < m) {
+        s_a[i] = a;
+        if (bin) atomicAdd(&s_hist[bin], 1u);
+      }
+      // exact zeros (untouched embedding rows) would all meet in one bin
+      const uint32_t zeros = __ballot_sync(0xffffffffu, i < m && bin == 0);
+      if (lane == 0 && zeros) atomicAdd(&s_hist[0], __popc(zeros));
+    }
+  }
+  // the threshold: magnitudes >= prefix << sh are taken, the last level's
+  // equal ones only up to the remaining rank
+  uint32_t prefix = 0, k_rem = k, n_in = d;
+  int sh = 31;
+  cluster.sync();  // every CTA's merged bins start at zero
+  for (int level = 0; level < 3 && k > 0 && n_in != k_rem; ++level) {
+    const int width = level == 0 ? 11 : 10;
+    const uint32_t nb = 1u << width;
+    sh -= width;
+    if (level > 0) {
+      for (uint32_t b = tid; b < nb; b += kSelThreads) s_hist[b] = 0;
+      __syncthreads();
+      for (uint32_t i = tid; i < m; i += kSelThreads) {
+        const uint32_t mg = __float_as_uint(s_a[i]) & 0x7fffffffu;
+        if ((mg >> (sh + width)) == prefix) atomicAdd(&s_hist[(mg >> sh) & (nb - 1)], 1u);
+      }
+      __syncthreads();
+    }
+    uint32_t* merged = cluster.map_shared_rank(&s_merged[level][0], 0);
+    for (uint32_t b = tid; b < nb; b += kSelThreads)
+      if (s_hist[b]) atomicAdd(merged + b, s_hist[b]);
+    cluster.sync();
+    for (uint32_t b = tid; b < nb; b += kSelThreads) s_hist[b] = merged[b];
+    __syncthreads();
+    const Selection s = select_bin<kSelThreads, false>(s_hist, nb, k_rem, s_w);
+    prefix = (prefix << width) | s.bin;  // found: the bins hold every value of the prefix
+    k_rem = s.k_rem;
+    n_in = s.n_in;
+  }
+  const bool ties = n_in != k_rem;  // at the last level (or k == 0: nothing is taken)
+  const uint32_t B = prefix << sh;
+  // this slice's counts: above the threshold and at it (with ties), or all taken
+  constexpr uint32_t kBlock = 4 * kSelThreads;  // positions per ordered round
+  uint32_t above = 0, equal = 0;
+  for (uint32_t i = tid; i < m; i += kSelThreads) {
+    const uint32_t mg = __float_as_uint(s_a[i]) & 0x7fffffffu;
+    above += (ties ? mg > B : mg >= B) ? 1u : 0u;
+    equal += ties && mg == B ? 1u : 0u;
+  }
+  if (k == 0) above = equal = 0;
+  uint32_t total;
+  block_exclusive<kSelThreads>(above, total, s_w);
+  if (tid == 0) s_above = total;
+  block_exclusive<kSelThreads>(equal, total, s_w);
+  if (tid == 0) s_equal = total;
+  cluster.sync();
+  uint32_t base = 0, eq_before = 0;  // pairs and equal magnitudes of the earlier slices
+  for (uint32_t q = 0; q < rank; ++q) {
+    base += *cluster.map_shared_rank(&s_above, q);
+    eq_before += *cluster.map_shared_rank(&s_equal, q);
+  }
+  const uint32_t most = ties && k > 0 ? k_rem : 0u;  // equal magnitudes taken in all
+  base += min(eq_before, most);
+  const uint32_t quota = most > eq_before ? most - eq_before : 0u;  // of this slice's
+  const bool vec = (reinterpret_cast<uintptr_t>(e) & 15u) == 0;     // (lo is a multiple of 4)
+  uint32_t seen_above = 0, seen_equal = 0;
+  ErrAcc acc;
+  for (uint32_t b0 = 0; b0 < m; b0 += kBlock) {
+    const uint32_t i0 = b0 + 4 * tid;
+    float a[4];
+    uint32_t up = 0, eq = 0;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      a[j] = i0 + j < m ? s_a[i0 + j] : 0.0f;
+      const uint32_t mg = __float_as_uint(a[j]) & 0x7fffffffu;
+      if (i0 + j < m && k > 0) {
+        up |= ((ties ? mg > B : mg >= B) ? 1u : 0u) << j;
+        eq |= (ties && mg == B ? 1u : 0u) << j;
+      }
+    }
+    const uint32_t before =
+        block_exclusive<kSelThreads>((__popc(eq) << 16) | __popc(up), total, s_w);
+    uint32_t n_up = seen_above + (before & 0xffffu), n_eq = seen_equal + (before >> 16);
+    seen_above += total & 0xffffu;
+    seen_equal += total >> 16;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      if (i0 + j >= m) continue;
+      const bool is_eq = (eq >> j) & 1u;
+      if (((up >> j) & 1u) || (is_eq && n_eq < quota)) {
+        const uint32_t pos = base + n_up + min(n_eq, quota);  // < k
+        idx_out[pos] = lo + i0 + j;
+        val_out[pos] = a[j];
+        a[j] = 0.0f;  // residual of a sent coordinate
+      } else if (err_out) {
+        acc.add(a[j]);
+      }
+      n_up += (up >> j) & 1u;
+      n_eq += is_eq ? 1u : 0u;
+    }
+    if (vec && i0 + 4 <= m) {
+      *reinterpret_cast<float4*>(e + lo + i0) = make_float4(a[0], a[1], a[2], a[3]);
+    } else {
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        if (i0 + j < m) e[lo + i0 + j] = a[j];
+    }
+  }
+  if (rank == 0 && tid == 0) *count_out = k;
+  if (err_out) {
+    acc.flush();
+    const FF share = block_sum_ff(acc.total, s_ff);
+    if (tid == 0) s_share = share;
+  }
+  cluster.sync();  // the counts are read, the shares are there
+  if (err_out) {
+    if (rank == 0 && tid == 0) {
+      FF sum{0.0f, 0.0f};
+      for (uint32_t q = 0; q < C; ++q) sum = ff_add(sum, *cluster.map_shared_rank(&s_share, q));
+      *err_out = ff_to_double(sum);
+    }
+    cluster.sync();  // no CTA leaves while its share is read
+  }
+}
+
+template <typename GT>
+cudaError_t launch_cluster(const GT* g, float* e, float gamma, uint32_t k, uint32_t d,
+                           uint32_t* idx_out, float* val_out, uint32_t* count_out,
+                           double* err_out, cudaStream_t stream) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(kClusterCtas);
+  cfg.blockDim = dim3(kSelThreads);
+  const uint32_t per = ((d + kClusterCtas - 1) / kClusterCtas + 3u) & ~3u;
+  cfg.dynamicSmemBytes = per * sizeof(float);
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = kClusterCtas;
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+  const cudaError_t err = cudaLaunchKernelEx(&cfg, topk_cluster_kernel<GT>, g, e, gamma, k, d,
+                                             idx_out, val_out, count_out, err_out);
+  count_launch();
+  return err;
+}
+
 template <typename GT, bool kAny>
 int tk_group_blocks_per_sm() {
   const void* fn = group_kernel<GT, kAny>();
@@ -1172,6 +1383,10 @@ void topk_init_device(DeviceInfo& info) {
   int a = 0;
   cudaFuncSetAttribute(topk_select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSelSmem);
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, topk_select_kernel, kSelThreads, kSelSmem);
+  cudaFuncSetAttribute(topk_cluster_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                       kClusterSmem);
+  cudaFuncSetAttribute(topk_cluster_kernel<uint16_t>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                       kClusterSmem);
   info.refine_blocks = a * info.sm_count;
   info.finalize_blocks = info.refine_blocks;
   info.tk_stream_per_sm_f32 =
@@ -1197,6 +1412,8 @@ cudaError_t launch_topk(const void* g, bool g_bf16, float* e, float gamma, uint3
                         uint32_t d, uint32_t* idx_out, float* val_out, uint32_t* count_out,
                         double* err_out, Workspace& ws, const DeviceInfo& dev) {
   auto run = [&](auto* gt) {
+    if (d <= kClusterMax && stream_kernel_mode() == 0)
+      return launch_cluster(gt, e, gamma, k, d, idx_out, val_out, count_out, err_out, ws.stream);
     return positions(gt, e).any() ? launch_typed<true>(gt, e, gamma, k, d, idx_out, val_out,
                                                        count_out, err_out, ws, dev)
                                   : launch_typed<false>(gt, e, gamma, k, d, idx_out, val_out,
