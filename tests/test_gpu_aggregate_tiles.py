@@ -61,6 +61,25 @@ def test_dense_sum_around_the_rule(d, n, tiles, off):
     assert efs.ef_check_status() == efs.EF_OK
 
 
+@pytest.mark.parametrize("n", [1, 31, 130, 256])
+@pytest.mark.parametrize("tiles", [1, 2, 911])
+def test_runs_searched_in_place(tiles, n):
+    # up to 911 tiles the reduction searches its runs: empty lists, runs that
+    # end with their list, lists that begin at a tile's edge, several hundred lists
+    d = tiles * TILE - (3 if tiles < 911 else 0)
+    rng = np.random.default_rng(n)
+    idx = []
+    for w in range(n):
+        j = rng.choice(d, min(d, [0, 1, 7, 300][w % 4]), replace=False)
+        if w % 4 == 2 and tiles > 1:
+            j = np.concatenate([j, [TILE - 1, TILE, d - 1]])
+        idx.append(np.unique(j).astype(np.uint32))
+    val = [rng.standard_normal(j.size).astype(np.float32) for j in idx]
+    gu.assert_bits(_sum(idx, val, d, False), oracle.sparse_aggregate(idx, val, d),
+                   "tiles=%d n=%d" % (tiles, n))
+    assert efs.ef_check_status() == efs.EF_OK
+
+
 def test_more_entries_than_the_scatter_takes():
     d, n = 1300 * TILE - 5, 3
     idx, val = _lists(d, [3_000_000] * n, 9)  # over 8 M entries: searches
