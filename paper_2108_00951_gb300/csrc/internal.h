@@ -15,8 +15,9 @@ namespace efs {
 constexpr size_t kOffBarGen = 0;        // uint32: grid-barrier generation (never reset)
 constexpr size_t kOffError = 8;         // uint32: latched device error bits
 constexpr size_t kOffBarArrive = 16;    // uint32: grid-barrier arrivals (zero after each barrier)
-constexpr size_t kOffTileClaim = 24;    // uint32[3]: work dispenser: handed out, CTAs finished,
-                                        // groups resolved (zero between calls)
+constexpr size_t kOffTileClaim = 24;    // uint32[4]: work dispenser: handed out, CTAs that take no
+                                        // more; and with an error norm groups resolved, CTAs
+                                        // finished (zero between calls)
 constexpr size_t kOffTkListCount = 72;  // uint32: candidates emitted by the streaming pass
 constexpr size_t kOffErrArrive = 80;    // uint32: arrivals of the e' norm pass (zero after it)
 constexpr size_t kOffRoundTotal = 84;   // uint32: coordinates the rounding did not send (zero after it)

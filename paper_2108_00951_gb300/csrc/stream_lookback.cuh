@@ -286,6 +286,12 @@ __global__ void __launch_bounds__(kLbThreads, 1)
         vst(s_cq_tail, ++tail);
         if (g >= G) break;
       }
+      // this CTA claims no more; the last to say so leaves the counter at zero
+      // for the next launch (here and not at the end: off the critical path)
+      if (atomicAdd(ctx.tile_claim + 1, 1u) == gridDim.x - 1) {
+        ctx.tile_claim[0] = 0;
+        ctx.tile_claim[1] = 0;
+      }
     }
     // ------------------------------------------------------ producer
     if (lane == 0) {
@@ -653,27 +659,23 @@ __global__ void __launch_bounds__(kLbThreads, 1)
     }
   }
 
-  // every CTA counts itself finished (after its resolved groups); the last
-  // one leaves the counters at zero for the next launch and, when every
-  // group was resolved, adds the groups' error shares
+  if (!la.err_out) return;
+  // every CTA counts itself finished, with its resolved groups; the last one
+  // adds the groups' error shares when every group was resolved
   __syncthreads();
-  uint32_t resolved_all = 0;
   if (threadIdx.x == 0) {
     atomicAdd(ctx.tile_claim + 2, s_resolved);
     __threadfence();
-    const uint32_t done = atomicAdd(ctx.tile_claim + 1, 1u);
-    s_last = done == gridDim.x - 1 ? 1u : 0u;
+    s_last = atomicAdd(ctx.tile_claim + 3, 1u) == gridDim.x - 1 ? 1u : 0u;
     if (s_last) {
       __threadfence();
-      resolved_all = atomicAdd(ctx.tile_claim + 2, 0u);
-      ctx.tile_claim[0] = 0;
-      ctx.tile_claim[1] = 0;
+      s_resolved = atomicAdd(ctx.tile_claim + 2, 0u);
       ctx.tile_claim[2] = 0;
-      s_resolved = resolved_all;
+      ctx.tile_claim[3] = 0;
     }
   }
   __syncthreads();
-  if (s_last && la.err_out) {
+  if (s_last) {
     __threadfence();
     const bool ok = s_resolved == G;
     const FF err = sum_parts_ff(la.err_parts, ok ? G : 0u, s_err_sum);
