@@ -193,8 +193,7 @@ cudaError_t launch_groups(const StreamIn<GT, kAny>& in, float gamma, float lambd
   const uint32_t grid = groups < slots ? groups : slots;
   uint32_t cap = d;
   ScanCtx c = ctx;
-  // the groups' shares of ||e'||^2 use the per-tile count area (16 words a tile)
-  LbArgs la{tiles_out, err_out, reinterpret_cast<FF*>(ws.counts()), ws.stage_pairs(), ws.density_dev};
+  LbArgs la = lb_args(ws, tiles_out, err_out, ws.density_dev);
   void* params[] = {&op, &idx_out, &val_out, &count_out, &cap, &c, &la};
   const cudaError_t err = launch_pdl(
       reinterpret_cast<const void*>(

@@ -15,8 +15,9 @@ namespace efs {
 constexpr size_t kOffBarGen = 0;        // uint32: grid-barrier generation (never reset)
 constexpr size_t kOffError = 8;         // uint32: latched device error bits
 constexpr size_t kOffBarArrive = 16;    // uint32: grid-barrier arrivals (zero after each barrier)
-constexpr size_t kOffTileClaim = 24;    // uint32[4]: work dispenser: handed out, CTAs that take no
-                                        // more; and with an error norm groups resolved, CTAs
+constexpr size_t kOffGroupClaim = 24;   // uint32[2]: groups handed out, by the parity of the
+                                        // claimed-group calls (each call zeroes the other)
+constexpr size_t kOffGroupErr = 32;     // uint32[2]: with an error norm: groups resolved, CTAs
                                         // finished (zero between calls)
 constexpr size_t kOffTkListCount = 72;  // uint32: candidates emitted by the streaming pass
 constexpr size_t kOffErrArrive = 80;    // uint32: arrivals of the e' norm pass (zero after it)
@@ -124,6 +125,7 @@ struct Workspace {
   size_t offsets_cap = 0;      // capacity of the aggregation offsets (uint32)
   size_t stage_cap = 0;        // capacity of the pair staging buffers (pairs)
   uint32_t epoch = 0;          // last epoch handed to a compaction launch
+  uint32_t group_calls = 0;    // claimed-group launches so far: their parity picks the counter
   uint32_t topk_calls = 0;     // Top-k calls so far: their parity picks the state block
   // Balanced chunks of the streaming hard-threshold kernel: each call computes
   // the next call's chunk boundaries from the previous call's chunk totals.

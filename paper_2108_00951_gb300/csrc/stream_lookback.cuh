@@ -72,6 +72,7 @@
 // depend on which CTA took which group.
 #pragma once
 
+#include "internal.h"
 #include "stream_compact.cuh"
 
 namespace efs {
@@ -134,11 +135,14 @@ struct LbLayout {
 };
 
 struct LbArgs {
+  uint32_t* claim;      // groups handed out so far, zero at the call's start
+  uint32_t* claim_next; // the next call's counter, zeroed here
   uint32_t* tile_base;  // optional [num_tiles + 1]: output position of each tile's first pair,
                         // and the total (untruncated), or null
   double* err_out;      // optional: sum of a^2 over the coordinates whose residual is final
                         // here (not selected, not deferred), or null
   FF* err_parts;        // [groups] the groups' shares of it (used when err_out is set)
+  uint32_t* err_count;  // [2] groups resolved, CTAs finished (zero between calls)
   uint2* slot;          // [num_tiles * 16 * 256] a segment's pairs (index, value bits) when its
                         // warp's buffer is full: segment (tile, warp) at (tile * 16 + warp) * 256
   uint32_t* density_out;  // optional (host-mapped): the call's pair count * 65536 / d, a hint
@@ -150,6 +154,15 @@ __device__ __forceinline__ uint32_t vld(const uint32_t& x) {
 }
 __device__ __forceinline__ void vst(uint32_t& x, uint32_t v) {
   *reinterpret_cast<volatile uint32_t*>(&x) = v;
+}
+
+// The arguments of a launch on a workspace (the groups' shares of ||e'||^2 use
+// the per-tile count area, 16 words a tile).
+inline LbArgs lb_args(Workspace& ws, uint32_t* tile_base, double* err_out, uint32_t* density_out) {
+  const uint32_t parity = ws.group_calls++ & 1u;
+  return LbArgs{ws.u32(kOffGroupClaim) + parity, ws.u32(kOffGroupClaim) + (parity ^ 1u), tile_base,
+                err_out, reinterpret_cast<FF*>(ws.counts()), ws.u32(kOffGroupErr),
+                ws.stage_pairs(), density_out};
 }
 
 // Bounded spin of one thread until pred() holds; false (and the CTA's failed
@@ -265,32 +278,40 @@ __global__ void __launch_bounds__(kLbThreads, 1)
         if (op.full(t)) op.prefetch(t);
       }
   }
-  // everything the previous kernels on the stream wrote (and the reset
-  // group counter) is read only after this
+  // The first claims too are made before the wait: this call's counter was
+  // left at zero by the call before on this workspace (each zeroes the other
+  // of two, whose user is complete by then, before it lets the next start).
+  const bool claimer = warp == kLbProducerWarp && lane == 1;
+  uint32_t claimed = 0;  // claimer: groups claimed so far, and whether that was all
+  bool last_claim = false;
+  if (claimer) {
+    for (; claimed < kLbClaimAhead && !last_claim; ++claimed) {
+      const uint32_t g = atomicAdd(la.claim, 1u);
+      s_cq[claimed] = g;
+      last_claim = g >= G;
+    }
+    __threadfence_block();
+    vst(s_cq_tail, claimed);
+  }
+  // everything the previous kernels on the stream wrote is read only after this
   griddep_wait();
   op.prologue();
   const uint64_t aux = op.initial_aux();  // uniform
 
   if (warp == kLbProducerWarp) {
-    if (lane == 1) {
+    if (claimer) {
       // ---------------------------------------------------- claimer
       // Claims groups up to kLbClaimAhead ahead of the producer, so that a
       // claim's round trip never stalls the producer's refills (a fence or
       // an mbarrier arrival of the producer would wait for it).
-      uint32_t tail = 0;
-      while (true) {
-        if (!lb_spin([&] { return tail - vld(s_cq_head) < kLbClaimAhead; }, &s_failed, ctx)) break;
-        const uint32_t g = atomicAdd(ctx.tile_claim, 1u);
-        s_cq[tail % kLbClaimAhead] = g;
+      while (!last_claim) {
+        if (!lb_spin([&] { return claimed - vld(s_cq_head) < kLbClaimAhead; }, &s_failed, ctx))
+          break;
+        const uint32_t g = atomicAdd(la.claim, 1u);
+        s_cq[claimed % kLbClaimAhead] = g;
         __threadfence_block();
-        vst(s_cq_tail, ++tail);
-        if (g >= G) break;
-      }
-      // this CTA claims no more; the last to say so leaves the counter at zero
-      // for the next launch (here and not at the end: off the critical path)
-      if (atomicAdd(ctx.tile_claim + 1, 1u) == gridDim.x - 1) {
-        ctx.tile_claim[0] = 0;
-        ctx.tile_claim[1] = 0;
+        vst(s_cq_tail, ++claimed);
+        last_claim = g >= G;
       }
     }
     // ------------------------------------------------------ producer
@@ -298,6 +319,10 @@ __global__ void __launch_bounds__(kLbThreads, 1)
       const uint64_t policy = l2_evict_normal_policy();
       uint32_t r = 0, seq = 0;
       bool ok = true;
+      if (blockIdx.x == 0) {
+        *la.claim_next = 0;
+        __threadfence();  // before this thread lets the next kernel be scheduled
+      }
       // the stage of use r is free once its previous use was released
       auto stage_free = [&](int s) {
         return r < static_cast<uint32_t>(kStages) ||
@@ -664,14 +689,14 @@ __global__ void __launch_bounds__(kLbThreads, 1)
   // adds the groups' error shares when every group was resolved
   __syncthreads();
   if (threadIdx.x == 0) {
-    atomicAdd(ctx.tile_claim + 2, s_resolved);
+    atomicAdd(la.err_count, s_resolved);
     __threadfence();
-    s_last = atomicAdd(ctx.tile_claim + 3, 1u) == gridDim.x - 1 ? 1u : 0u;
+    s_last = atomicAdd(la.err_count + 1, 1u) == gridDim.x - 1 ? 1u : 0u;
     if (s_last) {
       __threadfence();
-      s_resolved = atomicAdd(ctx.tile_claim + 2, 0u);
-      ctx.tile_claim[2] = 0;
-      ctx.tile_claim[3] = 0;
+      s_resolved = atomicAdd(la.err_count, 0u);
+      la.err_count[0] = 0;
+      la.err_count[1] = 0;
     }
   }
   __syncthreads();
