@@ -351,16 +351,30 @@ struct Source {
   bool list;
   uint32_t c0, n;
 };
-__device__ Source segment_source(const LwArgs& a, const LwSeg& s, uint32_t si) {
+// What the stream left about a segment: its bound and the list positions
+// around its ends, loaded in one round trip.
+struct SegHead {
+  uint32_t bound, p0, p1, q0, q1;
+};
+__device__ __forceinline__ SegHead segment_head(const LwArgs& a, const LwSeg& s, uint32_t si) {
+  const uint32_t tl =
+      static_cast<uint32_t>((static_cast<uint64_t>(s.lo) + a.shift) / kTileElems);  // < tiles
+  const uint32_t th =
+      static_cast<uint32_t>((static_cast<uint64_t>(s.hi) + a.shift) / kTileElems);  // <= tiles
+  SegHead h;
+  h.bound = __ldcg(a.mbound + si);
+  h.p0 = __ldcg(a.tile_base + tl);
+  h.p1 = __ldcg(a.tile_base + min(tl + 1, a.tiles));
+  h.q0 = __ldcg(a.tile_base + th);
+  h.q1 = __ldcg(a.tile_base + min(th + 1, a.tiles));
+  return h;
+}
+__device__ Source segment_source(const LwArgs& a, const LwSeg& s, const SegHead& h) {
   Source src{false, 0, s.hi - s.lo};
-  if (__ldcg(a.mbound + si) >= kLwDeferred) return src;
+  if (h.bound >= kLwDeferred) return src;
   const uint64_t p_lo = static_cast<uint64_t>(s.lo) + a.shift;
   const uint64_t p_hi = static_cast<uint64_t>(s.hi) + a.shift;
-  const uint32_t tl = static_cast<uint32_t>(p_lo / kTileElems);  // < tiles
-  const uint32_t th = static_cast<uint32_t>(p_hi / kTileElems);  // <= tiles
-  const uint32_t p0 = __ldcg(a.tile_base + tl), p1 = __ldcg(a.tile_base + tl + 1);
-  const uint32_t q0 = __ldcg(a.tile_base + th);
-  const uint32_t q1 = th < a.tiles ? __ldcg(a.tile_base + th + 1) : q0;
+  const uint32_t p0 = h.p0, p1 = h.p1, q0 = h.q0, q1 = h.q1;
   // candidates of the partial tiles that lie below lo / hi (none to scan
   // when lo / hi starts a tile); a tile cut off at the capacity disqualifies
   const uint32_t e0 = p_lo % kTileElems ? p1 : p0, e1 = p_hi % kTileElems ? q1 : q0;
@@ -546,14 +560,11 @@ struct NoTeam {
 // Where the streaming pass left a segment's residuals to the select: every
 // position of a list source (candidates), and of an e source those at or above
 // the bound the stream used (all of them without one).
-__device__ __forceinline__ uint32_t err_from_for(const LwArgs& a, const LwSeg& s, uint32_t si,
-                                                 bool list) {
-  if (list || s.kind != kLwSampled) return 0u;
-  const uint32_t b = __ldcg(a.mbound + si);
-  return b >= kLwDeferred ? 0u : b;
+__device__ __forceinline__ uint32_t err_from_for(const LwSeg& s, uint32_t bound, bool list) {
+  return list || s.kind != kLwSampled || bound >= kLwDeferred ? 0u : bound;
 }
 
-__device__ bool select_single(const LwArgs& a, const LwSeg& s, uint32_t si, float* e,
+__device__ bool select_single(const LwArgs& a, const LwSeg& s, const SegHead& head, float* e,
                               uint32_t* idx_out, float* val_out, bool& overflow,
                               uint32_t* s_bits, uint32_t* s_hist, uint32_t* s_w, uint32_t* s_lo,
                               uint32_t* s_hi, ErrAcc* err) {
@@ -568,8 +579,8 @@ __device__ bool select_single(const LwArgs& a, const LwSeg& s, uint32_t si, floa
     }
     return true;
   }
-  const Source src = s.kind == kLwWhole ? Source{false, 0, ds} : segment_source(a, s, si);
-  const uint32_t err_from = err_from_for(a, s, si, src.list);
+  const Source src = s.kind == kLwWhole ? Source{false, 0, ds} : segment_source(a, s, head);
+  const uint32_t err_from = err_from_for(s, head.bound, src.list);
   const float* vals = src.list ? a.list_val + src.c0 : e + s.lo;
   const uint32_t* idxs = src.list ? a.list_idx + src.c0 : nullptr;
   SmallSelection sel;
@@ -604,14 +615,15 @@ __device__ bool select_single(const LwArgs& a, const LwSeg& s, uint32_t si, floa
 // holding the cut publishes its position). The write-out scans per-rank
 // counts behind one more barrier. Returns false on a barrier that ran out
 // (latched as a timeout) or an inconsistent histogram.
-__device__ bool select_team(const LwArgs& a, const LwSeg& s, uint32_t si, uint32_t T, uint32_t r,
+__device__ bool select_team(const LwArgs& a, const LwSeg& s, const SegHead& head, uint32_t T,
+                            uint32_t r,
                             LwTeamState* st, float* e, uint32_t* idx_out, float* val_out,
                             bool& overflow, bool& bad, uint32_t* s_hist, uint32_t* s_w,
                             ErrAcc* err) {
   __shared__ uint32_t s_found, s_last;
   const int tid = threadIdx.x;
-  const Source src = segment_source(a, s, si);
-  const uint32_t err_from = err_from_for(a, s, si, src.list);
+  const Source src = segment_source(a, s, head);
+  const uint32_t err_from = err_from_for(s, head.bound, src.list);
   const float* vals = src.list ? a.list_val + src.c0 : e + s.lo;
   const uint32_t* idxs = src.list ? a.list_idx + src.c0 : nullptr;
   const MagsGlobal mag{vals};
@@ -740,11 +752,19 @@ __global__ void __launch_bounds__(kLwThreads, 1)
   __shared__ uint32_t s_w[kLwThreads / 32];
   __shared__ uint32_t s_lo[32], s_hi[32];
   const int tid = threadIdx.x;
+  // What the CTA selects first, from the plan's tables (copied to the device
+  // before this call's first kernel: nothing in flight writes them), while the
+  // stream pass ends.
+  const LwCta me = a.ctas[blockIdx.x];
+  const bool single = me.team == kLwNoTeam, idle = single && me.a >= me.b;
+  uint32_t si = idle ? 0u : single ? a.work_seg[me.a] : me.a;
+  LwSeg s = a.segs[si];
   // a dependent launch may start early: the stream pass's results are read
   // only after this; the next call's sampling may then be scheduled (it
   // writes nothing this kernel reads before waiting for it)
   griddep_wait();
   griddep_launch_dependents();
+  SegHead head = segment_head(a, s, si);
   const bool failed = (__ldcg(a.list_flags) & kDevErrTimeout) != 0;
   if (blockIdx.x == 0 && tid == 0) {
     *a.count_out = failed ? 0u : a.total_k;
@@ -757,19 +777,20 @@ __global__ void __launch_bounds__(kLwThreads, 1)
   bool overflow = false, bad = false;
   ErrAcc acc;
   ErrAcc* err = a.err_out ? &acc : nullptr;
-  const LwCta me = a.ctas[blockIdx.x];
-  if (me.team == kLwNoTeam) {
+  if (single) {
     for (uint32_t w = me.a; w < me.b; ++w) {
-      const uint32_t si = a.work_seg[w];
-      const LwSeg s = a.segs[si];
+      if (w > me.a) {
+        si = a.work_seg[w];
+        s = a.segs[si];
+        head = segment_head(a, s, si);
+      }
       __syncthreads();  // the previous segment is done with shared memory
-      if (!select_single(a, s, si, e, idx_out, val_out, overflow, s_bits, s_hist, s_w, s_lo,
+      if (!select_single(a, s, head, e, idx_out, val_out, overflow, s_bits, s_hist, s_w, s_lo,
                          s_hi, err))
         bad = true;
     }
   } else {
-    const LwSeg s = a.segs[me.a];
-    select_team(a, s, me.a, me.b, me.rank, a.teams + me.team, e, idx_out, val_out, overflow, bad,
+    select_team(a, s, head, me.b, me.rank, a.teams + me.team, e, idx_out, val_out, overflow, bad,
                 s_hist, s_w, err);
   }
   if (__syncthreads_or(overflow) && tid == 0) atomicOr(a.error, kDevErrOverflow);
