@@ -70,6 +70,7 @@ METRIC = "EF hard-threshold compress GB/s & elem/s vs HBM peak; Top-k and aggreg
 HT_KERNEL_SOURCES = ["paper_2108_00951_gb300/csrc/ht.cu",
                      "paper_2108_00951_gb300/csrc/stream_compact.cuh",
                      "paper_2108_00951_gb300/csrc/stream_lookback.cuh",
+                     "paper_2108_00951_gb300/csrc/stream_in.cuh",
                      "paper_2108_00951_gb300/csrc/tma.cuh",
                      "paper_2108_00951_gb300/csrc/compact.cuh",
                      "paper_2108_00951_gb300/csrc/common.cuh",
