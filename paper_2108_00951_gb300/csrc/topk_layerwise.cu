@@ -1078,7 +1078,12 @@ cudaError_t lw_prepare(Workspace& ws, const uint64_t* seg_end, const uint64_t* s
       const uint64_t sampled_groups = static_cast<uint64_t>(x.groups) * parts_of[s];
       const uint64_t est =
           x.exact ? x.k + 2048 : 3ull * x.k / 2 + 32ull * ds / (4ull * sampled_groups);
-      uint64_t want = est > kLwSmemElems * 3ull / 4 ? (est + 24575) / 24576 : 1;
+      // (a rank's passes over 8 K candidates take about as long as a team
+      // barrier: LSTM-shaped call at 1 %, an embedding with 281 K candidates, 127
+      // us with 24 K a rank, 109 with 8 K, 108 with 4 K and teams of up to 96,
+      // which take VGG-16's at 1 % from 413 to 666. Teams from 16 K or 24 K
+      // candidates on: ResNet-18 at 1 % 70 -> 64, but ResNet-50 113 -> 120 and 117)
+      uint64_t want = est > kLwSmemElems * 3ull / 4 ? (est + 8191) / 8192 : 1;
       // a segment one CTA would select slowly from e if its bound missed
       // gets a team, unless its merged sample makes a miss implausible
       if (parts_of[s] == 1) want = std::max<uint64_t>(want, (ds + (1u << 24) - 1) >> 24);
