@@ -459,9 +459,9 @@ void ef_test_set_lookback_fault(int64_t withheld_tile, uint32_t spin_limit_us);
  * hard-threshold step and of the Top-k and layer-wise Top-k candidate passes
  * (g and e at any alignment): 0 (the default) by size (claimed groups of tiles
  * with look-back from 4096 tiles, 16,777,216 coordinates, on; static chunks
- * below; for the hard-threshold step, a shallower ring with larger pair
- * buffers once an earlier call on the same stream sent at least 1/12 of its
- * coordinates), 1 static chunks, 2 claimed groups, 3 claimed groups with the
+ * below; for the hard-threshold step, once an earlier call on the same stream
+ * sent at least 1/12 of its coordinates, claimed groups from 1024 tiles on,
+ * with a shallower ring and larger pair buffers), 1 static chunks, 2 claimed groups, 3 claimed groups with the
  * shallower ring (hard-threshold; the candidate passes treat 3 as 2). With 0, a
  * Top-k call of at most 65,536 coordinates streams nothing: one thread-block
  * cluster does all of it. Any other value means 0. The results are the same

@@ -236,6 +236,7 @@ cudaError_t launch_chunks(const StreamIn<GT, kAny>& in, float gamma, float lambd
   sa.prev_part = same && ws.ht_prev_balanced ? ws.ht_part(seq + 2) : nullptr;  // seq - 1
   sa.prev_epoch = ws.ht_last_epoch;
   sa.part_out = ws.ht_part(seq + 1);
+  sa.density_out = ws.density_dev;
   void* params[] = {&op, &idx_out, &val_out, &count_out, &cap, &c, &sa};
   const cudaError_t err = launch_pdl(
       reinterpret_cast<const void*>(&stream_compact_kernel<HtOp<GT, kAny>, kHtStages<GT>>), grid,
@@ -265,11 +266,13 @@ cudaError_t launch_typed(const GT* g, float* e, float gamma, float lambda, uint3
   const int per_chunk = sizeof(GT) == 4 ? dev.ht_stream_per_sm_f32 : dev.ht_stream_per_sm_bf16;
   cudaError_t err = cudaErrorInvalidConfiguration;
   const int mode = stream_kernel_mode();
-  const bool groups = use_group_kernel(tiles) && per_group > 0;
-  const bool dense =
-      groups && per_dense > 0 &&
-      (mode == 3 || (mode == 0 && ws.density_host &&
-                     *static_cast<volatile uint32_t*>(ws.density_host) >= kDenseRingHint));
+  const bool dense_hint = mode == 0 && ws.density_host &&
+                          *static_cast<volatile uint32_t*>(ws.density_host) >= kDenseRingHint;
+  // (a norm's summation order is the kernel's: with one, the size alone decides)
+  const bool groups =
+      per_group > 0 && (use_group_kernel(tiles) ||
+                        (dense_hint && tiles >= kDenseGroupMinTiles && !err_out));
+  const bool dense = groups && per_dense > 0 && (mode == 3 || dense_hint);
   if (dense)
     err = launch_groups<kHtStages<GT> - 1>(in, gamma, lambda, d, idx_out, val_out, count_out,
                                                err_out, kernel_tiles, ws, dev, ctx, per_dense);

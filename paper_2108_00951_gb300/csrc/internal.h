@@ -267,6 +267,12 @@ inline bool use_group_kernel(uint32_t tiles) {
 // kernel with one ring stage fewer and the freed shared memory added to the
 // warps' pair buffers: fewer segments go through their global slots.
 constexpr uint32_t kDenseRingHint = 65536u / 12u;  // 8.3 %
+// Dense hard-threshold calls take the claimed-group kernel from this many tiles
+// on (4.2 M coordinates): the static chunks' placement of many pairs is what
+// ends a call. Measured on a GB300, us a call, static chunks -> claimed groups:
+// 10 % sent, d = 2 M 14.3 -> 15.5, 5 M 18.1 -> 17.4, 11 M 34.4 -> 30.4, 15 M 43.6 -> 39.3;
+// 20 % sent, 5 M 22.3 -> 18.8, 11 M 39.2 -> 33.2, 15 M 51.0 -> 41.3; at 5 % equal.
+constexpr uint32_t kDenseGroupMinTiles = 1024;
 ScanCtx next_scan_ctx(Workspace& ws, uint32_t num_tiles);
 
 // ---- launchers (return the launch's cudaError_t) ----

@@ -106,6 +106,8 @@ struct StreamArgs {
   const uint32_t* prev_part;  // the previous launch's boundaries (null: equal chunks)
   uint32_t prev_epoch;        // the previous launch's epoch
   uint32_t* part_out;         // [gridDim.x + 1] boundaries computed for the next launch
+  uint32_t* density_out;      // optional (host-mapped): the call's pairs * 65536 / d, a hint for
+                              // the host's choice of later calls' kernel, or null
 };
 
 // Weight of a chunk when the next launch's chunks are balanced: a coordinate
@@ -553,6 +555,9 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
   if (hi == T * kSWarps && threadIdx.x == 0) {
     *count_out = base < cap ? base : cap;
     if (sa.tile_base) sa.tile_base[T] = base;
+    if (sa.density_out)
+      *sa.density_out =
+          static_cast<uint32_t>((static_cast<uint64_t>(base) << 16) / (op.end - op.shift()));
   }
   if (__syncthreads_or(overflow) && threadIdx.x == 0) atomicOr(ctx.error, kDevErrOverflow);
 }
