@@ -13,8 +13,9 @@
 // (not needed when the messages come with their tile indexes); kernel 2 does
 // the reduction and writes each dense tile once with 16-byte stores: a CTA per
 // tile as above, or for a plain sum of up to 32 workers over many tiles one
-// warp per tile (agg_stream_kernel), where worker order needs no barriers. Traffic: 8 B per pair read + 4 B per coordinate
-// written (+ the small offsets table).
+// warp per tile (agg_stream_kernel), where worker order needs no barriers.
+// Traffic: 8 B per pair read + 4 B per coordinate written (+ the small offsets
+// table).
 //
 // The same reduction can instead end in the model update that follows the
 // exchange (sparse_aggregate_apply): Delta' = alpha * s rounded once, then

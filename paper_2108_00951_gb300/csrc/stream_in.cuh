@@ -25,8 +25,8 @@
 // Measured on a GB300 (LSTM-shaped vector, d = 28.9 M, 3 % sent, us per call):
 // rows 1..3 of [4, d] matrices (12, 8 and 4 bytes past a word) 280 with the
 // one-tile-per-CTA kernel that misaligned vectors used before, 66 for row 0;
-// here four such workers' calls and their exchange take 337 (991 before), the
-// alignment costing the streaming kernel nothing that shows.
+// four such workers' calls and their exchange went from 991 to 337 (and to 290
+// with what the exchange and the claimed-group kernel gained since).
 #pragma once
 
 #include "gradient.cuh"

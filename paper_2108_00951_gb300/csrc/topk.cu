@@ -628,7 +628,8 @@ __device__ void small_emit(const TopkArgs& args, float* e, uint32_t n, uint32_t 
 // The slices cost one round trip and the barriers two; the radix select below
 // reads the list five times around three to six barriers. Measured on a
 // GB300, LSTM-shaped call, k = 289 K of 28.9 M (0.45 M candidates): this
-// kernel 45 -> 28 us, the call 123 -> 103.5; ResNet-50-shaped, k = 1 %, 117 ->
+// kernel 45 -> 28 us, the call 123 -> 103.5 (99.4 with what the streaming
+// kernel gained since); ResNet-50-shaped, k = 1 %, 117 ->
 // 97; VGG-16-shaped, k = 1 %, 428 -> 358. Lists that one CTA holds stay with
 // it (ResNet-18-shaped, k = 0.1 %, 17 K candidates: 47.5 us a call, 57.8 this
 // way): its few CTAs let the next call's sampling start beside them. Returns false, uniformly over the grid, when it does not apply
