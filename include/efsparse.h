@@ -122,7 +122,9 @@ typedef enum {
  *                    coordinates, strictly ascending.
  *   val_out    [out] fp32[capacity >= d]; val_out[p] = a[idx_out[p]].
  *   count_out  [out] one uint32 in device memory: the number of pairs
- *                    (= ||C(a)||_0, the per-iteration k_t of Sec. 6).
+ *                    (= ||C(a)||_0, the per-iteration k_t of Sec. 6). After a
+ *                    step that failed on the device (a latched timeout) it is
+ *                    at most d and the lists hold no message.
  *   Outputs must not overlap g or e. Entries of idx_out/val_out at positions
  *   >= count are left untouched.
  */

@@ -57,7 +57,8 @@ struct AggPtrs {
 //    independent of the lists' length).
 // Either way every entry lies in [0, count]; a list that is not strictly
 // ascending is latched as bad input (scatter) and may leave entries the
-// reduction clamps to the list.
+// reduction clamps to the list. A strictly ascending list below d has at most
+// d entries: a larger count is latched, and nothing past d entries is read.
 // The scatter reads every index once (32 MB at most, about 8 us), the searches
 // take 8 to 12 us whatever the lists hold. Measured, us an exchange, searches
 // -> scatter: 16 lists of 256 K entries over 6,240 tiles 61.6 -> 54.8, 4
@@ -67,7 +68,8 @@ constexpr uint32_t kScatterEntries = 8u << 20;
 template <uint32_t kCap>
 __global__ void __launch_bounds__(kThreads)
     agg_offsets_kernel(AggPtrs<kCap> p, const uint32_t* __restrict__ counts, uint32_t n,
-                       uint32_t tiles, uint32_t* __restrict__ off, uint32_t* __restrict__ error) {
+                       uint32_t d, uint32_t tiles, uint32_t* __restrict__ off,
+                       uint32_t* __restrict__ error) {
   griddep_wait();                // the lists and counts come from the kernels before
   griddep_launch_dependents();    // the reduction may be scheduled (it waits for this grid)
   const uint32_t per = tiles + 1;
@@ -78,7 +80,8 @@ __global__ void __launch_bounds__(kThreads)
   uint32_t all = 0;  // entries of all lists (each clamped: 256 of them fit)
   for (uint32_t q = lane; q < n; q += 32) all += min(counts[q], 1u << 23);
   all = warp_sum(all);
-  const uint32_t cnt = counts[i];
+  const uint32_t cnt = min(counts[i], d);
+  if (counts[i] > d && tx == 0) atomicOr(error, kDevErrBadInput);
   const uint32_t* x = p.idx[i];
   uint32_t* o = off + static_cast<uint64_t>(i) * per;
   if (cnt < per / 16 || all > kScatterEntries) {
@@ -595,15 +598,15 @@ cudaError_t launch_reduce(bool vec, AggPtrs<kCap>& p, uint32_t n, uint32_t d, ui
 
 // Each list's position at every tile boundary, for lists without tile indexes.
 template <uint32_t kCap>
-cudaError_t launch_offsets(AggPtrs<kCap>& p, const uint32_t* counts, uint32_t n, uint32_t tiles,
-                           uint32_t* off, Workspace& ws) {
+cudaError_t launch_offsets(AggPtrs<kCap>& p, const uint32_t* counts, uint32_t n, uint32_t d,
+                           uint32_t tiles, uint32_t* off, Workspace& ws) {
   // a thread per tile for the searches; for the scatter about 8 CTAs per SM
   // in all, but no more than 16 entries a tile would occupy
   const uint32_t per_tile = (tiles + 1 + kThreads - 1) / kThreads;
   const uint32_t wide = std::min((1216 + n - 1) / n, (tiles / kThreads + 1) * 16);
   const dim3 grid(std::max(per_tile, wide), n);
   uint32_t* error = ws.u32(kOffError);
-  void* params[] = {&p, &counts, &n, &tiles, &off, &error};
+  void* params[] = {&p, &counts, &n, &d, &tiles, &off, &error};
   const cudaError_t err = launch_pdl(reinterpret_cast<const void*>(&agg_offsets_kernel<kCap>),
                                      grid, kThreads, 0, ws.stream, params, false);
   count_launch();
@@ -634,7 +637,7 @@ cudaError_t launch_common(uint32_t n, const uint32_t* const* idx, const float* c
   uint32_t* off = nullptr;
   if (!tile_index && tiles > kAggSearchTiles) {  // locate each list's tile boundaries first
     off = ws.offsets();
-    err = launch_offsets(p, counts, n, tiles, off, ws);
+    err = launch_offsets(p, counts, n, d, tiles, off, ws);
     if (err != cudaSuccess) return err;
   }
   const bool vec = reinterpret_cast<uintptr_t>(o.out) % 16 == 0 &&
@@ -727,7 +730,7 @@ cudaError_t launch_list_tiles(const uint32_t* idx, const uint32_t* count, uint32
                               uint32_t* tiles_out, Workspace& ws) {
   AggPtrs<kFewWorkers> p;
   p.idx[0] = idx;
-  return launch_offsets(p, count, 1, agg_tiles_for(d), tiles_out, ws);
+  return launch_offsets(p, count, 1, d, agg_tiles_for(d), tiles_out, ws);
 }
 
 }  // namespace efs

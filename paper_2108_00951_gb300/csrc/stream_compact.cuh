@@ -44,7 +44,8 @@
 // Traffic beyond the step itself: 16 bytes per selected pair (staging write
 // and read) plus 4 bytes per segment. Every wait (stage arrival, stage
 // release, an earlier chunk's total) is bounded and latches kDevErrTimeout;
-// after a timeout the CTA places no pair.
+// after a timeout the CTA places no pair, and the last chunk's writes a count
+// of 0.
 //
 // An Op supplies the per-segment work (on positions: coordinates plus
 // op.shift(); its inputs, from which it takes shift(), full(), fill(), prefetch()
@@ -369,13 +370,23 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
       if (static_cast<int64_t>(t) == ctx.withheld_tile) withheld = true;
     }
   }
+  // The CTA that would write the call's count says 0 when it stops early: what
+  // reads the message next (its tile index, the exchange) takes its length
+  // from there, and the word may hold anything before the call.
+  auto no_count = [&]() {
+    if (t_hi == T && threadIdx.x == 0) *count_out = 0;
+  };
   if (__syncthreads_or(failed)) {
     if (threadIdx.x == 0) atomicOr(ctx.error, kDevErrTimeout);
+    no_count();
     return;
   }
   // A CTA that owns the withheld tile never arrives: the others' barrier
   // waits run out (the failure-detection test).
-  if (__syncthreads_or(withheld)) return;
+  if (__syncthreads_or(withheld)) {
+    no_count();
+    return;
+  }
   griddep_launch_dependents();  // streaming is done: the next kernel may be scheduled
 
   // ------------------------------------------------------------- phase 2
@@ -481,6 +492,7 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
         const bool out_of_time = ++it > (1u << 26) || now - t0 > ctx.wait_limit_ns;
         if (__syncthreads_or(out_of_time)) {
           if (threadIdx.x == 0) atomicOr(ctx.error, kDevErrTimeout);
+          no_count();
           return;
         }
         __nanosleep(64);

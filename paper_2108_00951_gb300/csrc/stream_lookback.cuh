@@ -376,6 +376,7 @@ __global__ void __launch_bounds__(kLbThreads, 1)
     }
   } else if (warp == kLbScanWarp) {
     // ------------------------------------------------------ look-back
+    bool ended = false;  // at the end mark, and not at a wait that ran out
     for (uint32_t seq = 0;; ++seq) {
       const uint32_t slot = seq % kEntries;
       LbEntry& en = ent[slot];
@@ -384,6 +385,7 @@ __global__ void __launch_bounds__(kLbThreads, 1)
       const uint32_t g = en.group, nt = en.ntiles;
       if (nt == 0) {  // no more groups: the placers end too
         if (lane == 0) mbar_arrive(&s_ready[slot]);
+        ended = true;
         break;
       }
       // segment positions in (tile, warp) order: lane l holds segments
@@ -447,6 +449,12 @@ __global__ void __launch_bounds__(kLbThreads, 1)
         ++s_resolved;
       }
     }
+    // The last group's CTA writes the call's count, unless one of its waits
+    // runs out (or every CTA stops before that group is claimed). A CTA that
+    // stops says 0 instead: what reads the message next takes its length from
+    // that word, which may hold anything before the call. Where the count is
+    // written too, either of the two may stay; the call has failed.
+    if (!ended && lane == 0) *count_out = 0;
   } else if (warp == kLbAggWarp) {
     // ------------------------------------------------------ aggregates
     // Publishes each group's total as soon as its segments are counted (the

@@ -50,6 +50,33 @@ def test_lookback_wait_runs_out_and_recovers(method):
     _healthy_call_matches_oracle(g, e)
 
 
+@pytest.mark.usefixtures("stream_kernel")
+@pytest.mark.parametrize("e_off", [0, 1])
+def test_count_after_a_wait_that_ran_out(e_off):
+    # a failed call's count is 0 whatever the word held, so that nothing after
+    # it (with a shifted e the kernel that finds the tile index) reads past the
+    # lists
+    d = 40 * 4096 + 9
+    g, e = _inputs(d)
+    gd, ed = gu.to_dev(g, e_off), gu.to_dev(e, e_off)
+    idx = torch.zeros(d, dtype=torch.int32, device=gu.DEV)
+    val = torch.empty(d, device=gu.DEV)
+    cnt = torch.full((1,), 0x7fffffff, dtype=torch.int32, device=gu.DEV)
+    tiles = torch.full((efs.tiles_for(d),), -1, dtype=torch.int32, device=gu.DEV)
+    assert efs.ef_check_status() == efs.EF_OK
+    efs.ef_test_set_lookback_fault(5, 2000)
+    try:
+        efs.ef_hard_threshold(gd, ed, 0.1, 1e-3, idx, val, cnt, tiles_out=tiles)
+        status = efs.ef_check_status()
+    finally:
+        efs.ef_test_set_lookback_fault(-1)
+    assert status == efs.EF_ERR_TIMEOUT
+    assert int(cnt.item()) == 0
+    if e_off:
+        assert not tiles.any()
+    _healthy_call_matches_oracle(g, e)
+
+
 def test_aggregate_malformed_input_is_latched_not_faulting():
     d = 10_000
     good = np.array([1, 50, 9000], np.uint32)
