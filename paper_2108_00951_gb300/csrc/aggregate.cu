@@ -208,15 +208,20 @@ __global__ void __launch_bounds__(kThreads)
   }
   griddep_wait();  // the offsets (and everything before them) are complete
   griddep_launch_dependents();  // the next kernel waits for this grid before its reads
+  bool bad = false;
   if (search) {
-    // few tiles and no offsets: two threads per list search its run's ends
+    // few tiles and no offsets: two threads per list search its run's ends.
+    // The last tile's run ends with the list, so that indexes past every tile
+    // are in it, to be skipped and latched.
     for (uint32_t q0 = 0; q0 < 2 * n; q0 += kThreads) {
       const uint32_t q = q0 + threadIdx.x, i = q >> 1;
       uint32_t at = 0;
       if (i < n) {
         const uint64_t target = (static_cast<uint64_t>(t) + (q & 1u)) * kAggTile;
         const uint32_t* x = p.idx[i];
-        uint32_t hi = counts[i];
+        uint32_t hi = min(counts[i], d);  // a strictly ascending list holds no more
+        bad |= counts[i] > d;
+        if (t == tiles - 1 && (q & 1u)) at = hi;
         while (at < hi) {
           const uint32_t mid = at + (hi - at) / 2;
           if (static_cast<uint64_t>(__ldg(x + mid)) < target)
@@ -259,7 +264,6 @@ __global__ void __launch_bounds__(kThreads)
     if (lane == 0) s_pre[0] = 0;
   }
   __syncthreads();
-  bool bad = false;
   const uint32_t total = s_pre[n];
   // The tile's pairs of all workers, in worker order, a stage at a time:
   // every copy of a stage is in flight at once (one round trip), then the
@@ -288,7 +292,17 @@ __global__ void __launch_bounds__(kThreads)
       for (uint32_t q = a + threadIdx.x; q < z; q += kThreads) {
         const uint32_t j = st_idx[q];
         const uint64_t r = static_cast<uint64_t>(j) - j0;  // wraps when j < j0
-        if (r < kAggTile && j < d)
+        bool ok = r < kAggTile && j < d;
+        if (search) {
+          // nothing else has looked at the list: a run must ascend. (The pair
+          // before a run's first is below j0, or the search had gone on.)
+          const uint32_t at = b0 + q - s_pre[i];  // in the run
+          const uint32_t prev = q > a ? st_idx[q - 1]
+                                : at > 0 ? __ldg(p.idx[i] + s_lo[i] + at - 1) : j;
+          bad |= at > 0 && prev >= j;
+          ok &= at == 0 || prev != j;  // (two adds to one sum would race)
+        }
+        if (ok)
           acc[r] += st_val[q];
         else
           bad = true;  // unsorted or out-of-range input: skipped, latched

@@ -91,6 +91,57 @@ def test_aggregate_malformed_input_is_latched_not_faulting():
     _healthy_call_matches_oracle(g, e)
 
 
+def _long_run(at, fix):
+    """1,500 ascending entries of tile 1, one of them replaced: position 1,024
+    begins the second stage of the run."""
+    j = np.arange(4096, 4096 + 3000, 2)
+    j[at] = fix(j, at)
+    return j
+
+
+# every kind of malformed list in a call of its own, so that one kind's report
+# cannot stand in for another's: (name, the list, the coordinates it may touch)
+MALFORMED = [
+    ("past the last tile", lambda d: [2, 9, 4_000_000_000]),
+    ("at the last tile's end", lambda d: [2, -(-d // 4096) * 4096]),
+    ("past d in the last tile", lambda d: [2, d + 1]),
+    ("nothing but past d", lambda d: [4_000_000_000]),
+    ("another tile's, before it", lambda d: [5000, 10]),
+    ("descent within a tile", lambda d: [50, 40]),
+    ("repeat within a tile", lambda d: [50, 50]),
+    ("repeat across stages", lambda d: _long_run(1024, lambda j, a: j[a - 1])),
+    ("descent across stages", lambda d: _long_run(1024, lambda j, a: j[a - 1] - 1)),
+    ("repeat inside a stage", lambda d: _long_run(700, lambda j, a: j[a - 1])),
+]
+
+
+@pytest.mark.parametrize("update", [False, True])
+@pytest.mark.parametrize("d", [10_000, 911 * 4096 - 3])
+@pytest.mark.parametrize("bad", [m[1] for m in MALFORMED], ids=[m[0] for m in MALFORMED])
+def test_each_malformed_list_is_latched(bad, d, update):
+    good = np.array([1, 60, 9000], np.uint32)
+    lists = [good, np.asarray(bad(d), np.int64).astype(np.uint32)]
+    vals = [np.full(j.size, 2.0 + w, np.float32) for w, j in enumerate(lists)]
+    idx = [gu.to_dev(j.view(np.int32)) for j in lists]
+    val = [gu.to_dev(v) for v in vals]
+    counts = torch.tensor([j.size for j in lists], dtype=torch.int32, device=gu.DEV)
+    out = torch.zeros(d, device=gu.DEV)
+    assert efs.ef_check_status() == efs.EF_OK
+    if update:
+        efs.sparse_aggregate_apply(idx, val, counts, d, 1.0, out)
+    else:
+        efs.sparse_aggregate(idx, val, counts, d, out)
+    assert efs.ef_check_status() == efs.EF_ERR_BAD_INPUT
+    assert efs.ef_check_status() == efs.EF_OK
+    want = np.zeros(d, np.float32)
+    want[good] = 2.0
+    apart = np.ones(d, bool)               # coordinates the malformed list does not name
+    apart[lists[1][lists[1] < d]] = False
+    got = out.cpu().numpy() * (-1.0 if update else 1.0)
+    gu.assert_bits((got + 0.0)[apart], want[apart], "the other coordinates")
+    assert np.all(np.isfinite(got))
+
+
 def test_invalid_arguments_launch_nothing():
     before = efs.ef_kernel_launches()
     x = torch.zeros(100, device=gu.DEV)
