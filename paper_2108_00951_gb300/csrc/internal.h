@@ -8,6 +8,7 @@
 #include <cuda_runtime.h>
 
 #include "common.cuh"
+#include "lw_share.h"
 
 namespace efs {
 
@@ -81,7 +82,6 @@ struct LwSeg {      // one segment (device and host layout, 32 bytes)
 // (team == kLwNoTeam), or member `rank` of a team of b CTAs that selects
 // segment a together (team = the team's index).
 constexpr uint32_t kLwNoTeam = 0xffffffffu;
-constexpr uint32_t kLwMaxTeam = 32;
 struct LwCta {
   uint32_t team, a, b, rank;
 };

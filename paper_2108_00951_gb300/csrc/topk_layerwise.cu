@@ -841,6 +841,8 @@ int lw_stream_blocks_per_sm() {
   return n;
 }
 
+static_assert(kLwTeamFrom == kLwSmemElems * 3 / 4, "candidates that one CTA takes");
+
 size_t align256(size_t x) { return (x + 255) & ~static_cast<size_t>(255); }
 
 // Work estimate of a segment's selection by one CTA, in positions handled.
@@ -1063,58 +1065,39 @@ cudaError_t lw_prepare(Workspace& ws, const uint64_t* seg_end, const uint64_t* s
   // Select work. A segment whose candidates may exceed one CTA's shared
   // memory, or whose own length would make a selection from e slow for one
   // CTA, gets a team of co-resident CTAs; the others go, longest first, onto
-  // the least loaded of the remaining CTAs. At most sm_count x (select CTAs
-  // per SM) CTAs in all, so that the cooperative launch is resident.
+  // the least loaded of the remaining CTAs (lw_share.h). At most sm_count x
+  // (select CTAs per SM) CTAs in all, so that the cooperative launch is
+  // resident.
   const uint32_t budget =
       static_cast<uint32_t>(std::max(1, dev.sm_count * std::max(1, dev.lw_select_per_sm)));
-  std::vector<uint32_t> team_seg, team_size, singles;
+  std::vector<uint32_t> team_seg, team_size, singles, selecting;
+  std::vector<LwWork> work;
   for (uint32_t s = 0; s < n_seg; ++s) {
     const LwSeg& x = segs[s];
     if (x.kind == kLwNone) continue;
-    uint32_t t = 1;
+    LwWork w{0, select_cost(x), 1};
     if (x.kind == kLwSampled) {
       // candidates the bound aims at: 1.5 k_s, plus 32 samples' worth
       const uint64_t ds = x.hi - x.lo;
       const uint64_t sampled_groups = static_cast<uint64_t>(x.groups) * parts_of[s];
-      const uint64_t est =
-          x.exact ? x.k + 2048 : 3ull * x.k / 2 + 32ull * ds / (4ull * sampled_groups);
-      // (a rank's passes over 8 K candidates take about as long as a team
-      // barrier: LSTM-shaped call at 1 %, an embedding with 281 K candidates, 127
-      // us with 24 K a rank, 109 with 8 K, 108 with 4 K and teams of up to 96,
-      // which take VGG-16's at 1 % from 413 to 666. Teams from 16 K or 24 K
-      // candidates on: ResNet-18 at 1 % 70 -> 64, but ResNet-50 113 -> 120 and 117)
-      uint64_t want = est > kLwSmemElems * 3ull / 4 ? (est + 8191) / 8192 : 1;
+      w.candidates = x.exact ? x.k + 2048 : 3ull * x.k / 2 + 32ull * ds / (4ull * sampled_groups);
       // a segment one CTA would select slowly from e if its bound missed
       // gets a team, unless its merged sample makes a miss implausible
-      if (parts_of[s] == 1) want = std::max<uint64_t>(want, (ds + (1u << 24) - 1) >> 24);
-      t = static_cast<uint32_t>(std::min<uint64_t>(want, kLwMaxTeam));
+      if (parts_of[s] == 1) w.least = static_cast<uint32_t>((ds + (1u << 24) - 1) >> 24);
     }
-    if (t > 1) {
-      team_seg.push_back(s);
-      team_size.push_back(t);
-    } else {
-      singles.push_back(s);
-    }
+    selecting.push_back(s);
+    work.push_back(w);
   }
-  {
-    // shrink the teams until they leave at least one CTA for the singles
-    const uint32_t reserve = singles.empty() ? 0u : 1u;
-    uint64_t sum = 0;
-    for (uint32_t t : team_size) sum += t;
-    while (sum + reserve > budget) {
-      auto it = std::max_element(team_size.begin(), team_size.end());
-      if (*it <= 1) break;
-      --*it;
-      --sum;
-    }
-    for (size_t q = 0; q < team_seg.size();) {  // a team of one is a single
-      if (team_size[q] <= 1) {
-        singles.push_back(team_seg[q]);
-        team_seg.erase(team_seg.begin() + q);
-        team_size.erase(team_size.begin() + q);
-      } else {
-        ++q;
-      }
+  std::vector<uint32_t> share;
+  uint64_t candidates = 0;
+  for (const LwWork& w : work) candidates += w.candidates;
+  lw_share(work, budget, candidates > topk_candidate_capacity(d), share);
+  for (size_t q = 0; q < selecting.size(); ++q) {
+    if (share[q] > 1) {
+      team_seg.push_back(selecting[q]);
+      team_size.push_back(share[q]);
+    } else {
+      singles.push_back(selecting[q]);
     }
   }
   uint32_t team_ctas = 0;
