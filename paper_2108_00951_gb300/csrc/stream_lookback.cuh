@@ -454,7 +454,8 @@ __global__ void __launch_bounds__(kLbThreads, 1)
     // stops says 0 instead: what reads the message next takes its length from
     // that word, which may hold anything before the call. Where the count is
     // written too, either of the two may stay; the call has failed.
-    if (!ended && lane == 0) *count_out = 0;
+    if constexpr (!Op::kKeepPairs)
+      if (!ended && lane == 0) *count_out = 0;
   } else if (warp == kLbAggWarp) {
     // ------------------------------------------------------ aggregates
     // Publishes each group's total as soon as its segments are counted (the
