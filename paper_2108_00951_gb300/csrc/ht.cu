@@ -193,9 +193,11 @@ cudaError_t launch_groups(const StreamIn<GT, kAny>& in, float gamma, float lambd
   const uint32_t grid = groups < slots ? groups : slots;
   uint32_t cap = d;
   ScanCtx c = ctx;
-  LbArgs la = lb_args(ws, tiles_out, err_out, ws.density_dev);
+  LbArgs la;
+  cudaError_t err = lb_args(ws, tiles_out, err_out, ws.density_dev, &la);
+  if (err != cudaSuccess) return err;
   void* params[] = {&op, &idx_out, &val_out, &count_out, &cap, &c, &la};
-  const cudaError_t err = launch_pdl(
+  err = launch_pdl(
       reinterpret_cast<const void*>(
           &lookback_stream_kernel<HtOp<GT, kAny>, kStages, kHtEntries<GT, kStages>>),
       grid, kLbThreads, HtGroupKernel<GT, kAny, kStages>::kSmem, ws.stream, params, false);

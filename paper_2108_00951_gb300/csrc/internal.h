@@ -20,6 +20,7 @@ constexpr size_t kOffGroupClaim = 24;   // uint32[2]: groups handed out, by the 
                                         // claimed-group calls (each call zeroes the other)
 constexpr size_t kOffGroupErr = 32;     // uint32[2]: with an error norm: groups resolved, CTAs
                                         // finished (zero between calls)
+constexpr size_t kOffGroupCaptured = 40;  // uint32: groups handed out, of captured calls
 constexpr size_t kOffTkListCount = 72;  // uint32: candidates emitted by the streaming pass
 constexpr size_t kOffErrArrive = 80;    // uint32: arrivals of the e' norm pass (zero after it)
 constexpr size_t kOffRoundTotal = 84;   // uint32: coordinates the rounding did not send (zero after it)

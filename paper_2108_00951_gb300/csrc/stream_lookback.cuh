@@ -136,7 +136,7 @@ struct LbLayout {
 
 struct LbArgs {
   uint32_t* claim;      // groups handed out so far, zero at the call's start
-  uint32_t* claim_next; // the next call's counter, zeroed here
+  uint32_t* claim_next; // the next call's counter, zeroed here (null: a captured call's)
   uint32_t* tile_base;  // optional [num_tiles + 1]: output position of each tile's first pair,
                         // and the total (untruncated), or null
   double* err_out;      // optional: sum of a^2 over the coordinates whose residual is final
@@ -157,12 +157,27 @@ __device__ __forceinline__ void vst(uint32_t& x, uint32_t v) {
 }
 
 // The arguments of a launch on a workspace (the groups' shares of ||e'||^2 use
-// the per-tile count area, 16 words a tile).
-inline LbArgs lb_args(Workspace& ws, uint32_t* tile_base, double* err_out, uint32_t* density_out) {
-  const uint32_t parity = ws.group_calls++ & 1u;
-  return LbArgs{ws.u32(kOffGroupClaim) + parity, ws.u32(kOffGroupClaim) + (parity ^ 1u), tile_base,
-                err_out, reinterpret_cast<FF*>(ws.counts()), ws.u32(kOffGroupErr),
-                ws.stage_pairs(), density_out};
+// the per-tile count area, 16 words a tile). The two counters rely on every
+// launch running in the order it was made. A captured one may run later or
+// never: it takes a third, zeroed by a node of its own graph, and leaves the
+// order of the two as it is.
+inline cudaError_t lb_args(Workspace& ws, uint32_t* tile_base, double* err_out,
+                           uint32_t* density_out, LbArgs* la) {
+  uint32_t* const claims = ws.u32(kOffGroupClaim);
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  cudaError_t err = cudaStreamIsCapturing(ws.stream, &capture);
+  if (err != cudaSuccess) return err;
+  *la = LbArgs{nullptr, nullptr, tile_base, err_out, reinterpret_cast<FF*>(ws.counts()),
+               ws.u32(kOffGroupErr), ws.stage_pairs(), density_out};
+  if (capture == cudaStreamCaptureStatusNone) {
+    const uint32_t parity = ws.group_calls++ & 1u;
+    la->claim = claims + parity;
+    la->claim_next = claims + (parity ^ 1u);
+  } else {
+    la->claim = ws.u32(kOffGroupCaptured);
+    err = cudaMemsetAsync(la->claim, 0, sizeof(uint32_t), ws.stream);
+  }
+  return err;
 }
 
 // Bounded spin of one thread until pred() holds; false (and the CTA's failed
@@ -280,7 +295,8 @@ __global__ void __launch_bounds__(kLbThreads, 1)
   }
   // The first claims too are made before the wait: this call's counter was
   // left at zero by the call before on this workspace (each zeroes the other
-  // of two, whose user is complete by then, before it lets the next start).
+  // of two, whose user is complete by then, before it lets the next start); a
+  // captured call's by the memset before it.
   const bool claimer = warp == kLbProducerWarp && lane == 1;
   uint32_t claimed = 0;  // claimer: groups claimed so far, and whether that was all
   bool last_claim = false;
@@ -319,7 +335,7 @@ __global__ void __launch_bounds__(kLbThreads, 1)
       const uint64_t policy = l2_evict_normal_policy();
       uint32_t r = 0, seq = 0;
       bool ok = true;
-      if (blockIdx.x == 0) {
+      if (blockIdx.x == 0 && la.claim_next) {
         *la.claim_next = 0;
         __threadfence();  // before this thread lets the next kernel be scheduled
       }

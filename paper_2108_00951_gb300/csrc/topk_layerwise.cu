@@ -905,7 +905,9 @@ cudaError_t launch_typed(const GT* g, float* e, float gamma, uint32_t d, uint32_
     const uint32_t groups = (tiles + kLbGroupTiles - 1) / kLbGroupTiles;
     const uint32_t gslots = static_cast<uint32_t>(per_sm_groups * dev.sm_count);
     const uint32_t ggrid = groups < gslots ? groups : gslots;
-    LbArgs la = lb_args(ws, tile_base, err_out ? ws.stream_err() : nullptr, nullptr);
+    LbArgs la;
+    err = lb_args(ws, tile_base, err_out ? ws.stream_err() : nullptr, nullptr, &la);
+    if (err != cudaSuccess) return err;
     void* gp[] = {&op, &list_idx, &list_val, &list_count, &cap, &ctx, &la};
     err = launch_pdl(group_kernel<GT, kAny>(), ggrid, kLbThreads, GroupLayout<GT, kAny>::kSmem,
                      ws.stream, gp, false);
