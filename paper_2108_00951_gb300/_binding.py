@@ -109,13 +109,17 @@ def status_string(status: int) -> str:
 # Measured on the Grace host of a GB300, us a call, before -> after:
 # ef_hard_threshold 11.2 -> 5.6 (2.6 of it the library), sparse_aggregate of 4
 # lists 18.6 -> 11.
+# (A torch without CUDA has neither of the two functions; its tensors are
+# refused before a stream is asked for.)
 _Tensor = torch.Tensor
-_raw_stream = torch._C._cuda_getCurrentRawStream
-_current_device = torch._C._cuda_getDevice
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_current_device = getattr(torch._C, "_cuda_getDevice", None)
 
 
 def _stream(stream):
     if stream is None:
+        if _raw_stream is None or _current_device is None:
+            return torch.cuda.current_stream().cuda_stream
         return _raw_stream(_current_device())
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
