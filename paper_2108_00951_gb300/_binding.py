@@ -163,6 +163,12 @@ def _pointers(tensors, name, dtype, numel=0):
     return (ctypes.c_void_p * max(len(p), 1))(*p)
 
 
+def _real(x):
+    """x for a c_float parameter; what is no number is a TypeError here (in a
+    call's arguments ctypes makes it an ArgumentError)."""
+    return x if type(x) is float else ctypes.c_float(x)
+
+
 def _gradient(g: torch.Tensor):
     if g.dtype is torch.float32:
         return False
@@ -200,7 +206,7 @@ def ef_hard_threshold(g, e, gamma, lam, idx_out, val_out, count_out, stream=None
     d = e.numel()
     if g.numel() != d:
         raise ValueError("g and e differ in length")
-    head = (_dev(g, "g", g.dtype), _dev(e, "e", torch.float32), gamma, lam, d,
+    head = (_dev(g, "g", g.dtype), _dev(e, "e", torch.float32), _real(gamma), _real(lam), d,
             _dev(idx_out, "idx_out", torch.int32, d),
             _dev(val_out, "val_out", torch.float32, d),
             _dev(count_out, "count_out", torch.int32, 1))
@@ -225,7 +231,7 @@ def ef_topk(g, e, gamma, k, idx_out, val_out, count_out, stream=None, err_sq_out
     d = e.numel()
     if g.numel() != d:
         raise ValueError("g and e differ in length")
-    head = (_dev(g, "g", g.dtype), _dev(e, "e", torch.float32), gamma, int(k), d,
+    head = (_dev(g, "g", g.dtype), _dev(e, "e", torch.float32), _real(gamma), int(k), d,
             _dev(idx_out, "idx_out", torch.int32, k),
             _dev(val_out, "val_out", torch.float32, k),
             _dev(count_out, "count_out", torch.int32, 1))
@@ -255,7 +261,7 @@ def ef_topk_layerwise(g, e, gamma, seg_end, seg_k, idx_out, val_out, count_out, 
     if ends.ndim != 1 or ks.shape != ends.shape:
         raise ValueError("seg_end and seg_k must be 1-D of one length")
     total = int(ks.sum()) if ks.size else 0
-    head = (_dev(g, "g", g.dtype), _dev(e, "e", torch.float32), gamma, ends.size,
+    head = (_dev(g, "g", g.dtype), _dev(e, "e", torch.float32), _real(gamma), ends.size,
             ends.ctypes.data, ks.ctypes.data, d, _dev(idx_out, "idx_out", torch.int32, total),
             _dev(val_out, "val_out", torch.float32, total),
             _dev(count_out, "count_out", torch.int32, 1))
@@ -310,8 +316,8 @@ def sparse_aggregate_apply(idx_list, val_list, counts, d, alpha, x, m=None, mome
     idx_arr = _pointers(idx_list, "idx", torch.int32)
     val_arr = _pointers(val_list, "val", torch.float32)
     m_ptr = None if m is None else _dev(m, "m", torch.float32, d)
-    tail = (_dev(counts, "counts", torch.int32, n), int(d), alpha,
-            _dev(x, "x", torch.float32, d), m_ptr, momentum, lr, _stream(stream))
+    tail = (_dev(counts, "counts", torch.int32, n), int(d), _real(alpha),
+            _dev(x, "x", torch.float32, d), m_ptr, _real(momentum), _real(lr), _stream(stream))
     if tiles is not None:
         _check(lib.sparse_aggregate_apply_tiled(n, idx_arr, val_arr, _tile_array(tiles, n, d),
                                                 *tail), "sparse_aggregate_apply_tiled")
@@ -329,7 +335,7 @@ def ef_scaled_round(g, e, gamma, scale_log2, q_out, unsent_out, stream=None, err
     if g.numel() != d:
         raise ValueError("g and e differ in length")
     _check(lib.ef_scaled_round_ex(_dev(g, "g", g.dtype), int(bf16), _dev(e, "e", torch.float32),
-                                  gamma, int(scale_log2), d,
+                                  _real(gamma), int(scale_log2), d,
                                   _dev(q_out, "q_out", torch.int32, d),
                                   _dev(unsent_out, "unsent_out", torch.int32, 1),
                                   _err(err_sq_out), _stream(stream)), "ef_scaled_round_ex")
