@@ -184,11 +184,17 @@ __device__ __forceinline__ void prefetch_l2_bulk(const void* p, uint32_t bytes) 
   asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
 }
 
-template <bool kVec, int kMode, uint32_t kCap>
+// kSearch: without offsets or tile indexes, for few tiles (kAggSearchTiles). A
+// kernel of its own: with a run-time choice the check of the runs' order in
+// the adding loop cost the others too (64 lists of 140 K pairs, d = 138.4 M, 655
+// -> 685 us). It checks a stage at once: 64 lists of 1 %, d = 3.7 M, update,
+// take 67.1 us without the check, 70.2 this way, 74.3 with it in the loop that
+// adds worker by worker.
+template <bool kVec, int kMode, uint32_t kCap, bool kSearch>
 __global__ void __launch_bounds__(kThreads)
     agg_reduce_kernel(AggPtrs<kCap> p, uint32_t n, uint32_t d, uint32_t tiles,
                       const uint32_t* __restrict__ off, const uint32_t* __restrict__ counts,
-                      AggOut o, uint32_t* __restrict__ error, bool search) {
+                      AggOut o, uint32_t* __restrict__ error) {
   __shared__ __align__(16) float acc[kAggTile];
   __shared__ uint32_t s_lo[kCap], s_pre[kCap + 1];
   __shared__ uint32_t st_idx[kAggStage];
@@ -209,10 +215,10 @@ __global__ void __launch_bounds__(kThreads)
   griddep_wait();  // the offsets (and everything before them) are complete
   griddep_launch_dependents();  // the next kernel waits for this grid before its reads
   bool bad = false;
-  if (search) {
-    // few tiles and no offsets: two threads per list search its run's ends.
-    // The last tile's run ends with the list, so that indexes past every tile
-    // are in it, to be skipped and latched.
+  if constexpr (kSearch) {
+    // two threads per list search its run's ends. The last tile's run ends
+    // with the list, so that indexes past every tile are in it, to be skipped
+    // and latched.
     for (uint32_t q0 = 0; q0 < 2 * n; q0 += kThreads) {
       const uint32_t q = q0 + threadIdx.x, i = q >> 1;
       uint32_t at = 0;
@@ -271,18 +277,37 @@ __global__ void __launch_bounds__(kThreads)
   // each coordinate receives its contributions in worker order.
   for (uint32_t b0 = 0; b0 < total; b0 += kAggStage) {
     const uint32_t bn = total - b0 < kAggStage ? total - b0 : kAggStage;
+    uint32_t inner = 0;  // kSearch: bit per pair of the thread: not a run's first
+    uint32_t before = 0;  // thread 0: the index before the stage's first, of the same run
     {
-      uint32_t i = 0;
+      uint32_t i = 0, bit = 1;
       for (uint32_t q = threadIdx.x; q < bn; q += kThreads) {
         const uint32_t gp = b0 + q;
         while (s_pre[i + 1] <= gp) ++i;
         const uint32_t src = s_lo[i] + (gp - s_pre[i]);
         cp_async_4(st_idx + q, p.idx[i] + src);
         cp_async_4(st_val + q, p.val[i] + src);
+        if constexpr (kSearch) {
+          if (gp > s_pre[i]) {
+            inner |= bit;
+            if (q == 0) before = __ldg(p.idx[i] + src - 1);
+          }
+          bit <<= 1;
+        }
       }
     }
     cp_async_wait_all();
     __syncthreads();
+    if constexpr (kSearch) {
+      // nothing else has looked at the lists: a run must ascend. (The index
+      // before a run's first is below j0, or the search had gone on.)
+#pragma unroll
+      for (uint32_t u = 0; u < kAggStage / kThreads; ++u) {
+        const uint32_t q = u * kThreads + threadIdx.x;
+        const uint32_t prev = q > 0 ? st_idx[q - 1] : before;
+        bad |= ((inner >> u) & 1u) && prev >= st_idx[q];
+      }
+    }
     uint32_t i = 0;
     while (s_pre[i + 1] <= b0) ++i;  // the stage's first worker (uniform)
     for (; i < n && s_pre[i] < b0 + bn; ++i) {
@@ -292,17 +317,7 @@ __global__ void __launch_bounds__(kThreads)
       for (uint32_t q = a + threadIdx.x; q < z; q += kThreads) {
         const uint32_t j = st_idx[q];
         const uint64_t r = static_cast<uint64_t>(j) - j0;  // wraps when j < j0
-        bool ok = r < kAggTile && j < d;
-        if (search) {
-          // nothing else has looked at the list: a run must ascend. (The pair
-          // before a run's first is below j0, or the search had gone on.)
-          const uint32_t at = b0 + q - s_pre[i];  // in the run
-          const uint32_t prev = q > a ? st_idx[q - 1]
-                                : at > 0 ? __ldg(p.idx[i] + s_lo[i] + at - 1) : j;
-          bad |= at > 0 && prev >= j;
-          ok &= at == 0 || prev != j;  // (two adds to one sum would race)
-        }
-        if (ok)
+        if (r < kAggTile && j < d)
           acc[r] += st_val[q];
         else
           bad = true;  // unsorted or out-of-range input: skipped, latched
@@ -599,14 +614,20 @@ __global__ void __launch_bounds__(32)
   if (bad) atomicOr(error, kDevErrBadInput);
 }
 
+template <int kMode, uint32_t kCap, bool kSearch>
+const void* reduce_kernel(bool vec) {
+  return vec ? reinterpret_cast<const void*>(&agg_reduce_kernel<true, kMode, kCap, kSearch>)
+             : reinterpret_cast<const void*>(&agg_reduce_kernel<false, kMode, kCap, kSearch>);
+}
+
 template <int kMode, uint32_t kCap>
 cudaError_t launch_reduce(bool vec, AggPtrs<kCap>& p, uint32_t n, uint32_t d, uint32_t tiles,
                           const uint32_t* off, const uint32_t* counts, AggOut o, Workspace& ws) {
   uint32_t* error = ws.u32(kOffError);
-  bool search = !off && !p.tiles[0];
-  void* params[] = {&p, &n, &d, &tiles, &off, &counts, &o, &error, &search};
-  const void* fn = vec ? reinterpret_cast<const void*>(&agg_reduce_kernel<true, kMode, kCap>)
-                       : reinterpret_cast<const void*>(&agg_reduce_kernel<false, kMode, kCap>);
+  void* params[] = {&p, &n, &d, &tiles, &off, &counts, &o, &error};
+  const bool search = !off && !p.tiles[0];
+  const void* fn = search ? reduce_kernel<kMode, kCap, true>(vec)
+                          : reduce_kernel<kMode, kCap, false>(vec);
   return launch_pdl(fn, tiles, kThreads, 0, ws.stream, params, false);
 }
 
@@ -690,17 +711,14 @@ cudaError_t launch_any(uint32_t n, const uint32_t* const* idx, const float* cons
                                                        agg_stream_slots);
 }
 
-template <uint32_t kCap>
+template <uint32_t kCap, bool kSearch>
 void prefer_shared() {
-  const void* fns[] = {reinterpret_cast<const void*>(&agg_reduce_kernel<true, kAggDense, kCap>),
-                       reinterpret_cast<const void*>(&agg_reduce_kernel<false, kAggDense, kCap>),
-                       reinterpret_cast<const void*>(&agg_reduce_kernel<true, kAggSgd, kCap>),
-                       reinterpret_cast<const void*>(&agg_reduce_kernel<false, kAggSgd, kCap>),
-                       reinterpret_cast<const void*>(&agg_reduce_kernel<true, kAggMomentum, kCap>),
-                       reinterpret_cast<const void*>(&agg_reduce_kernel<false, kAggMomentum, kCap>)};
-  for (const void* f : fns)
-    cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout,
-                         cudaSharedmemCarveoutMaxShared);
+  for (bool vec : {false, true})
+    for (const void* f :
+         {reduce_kernel<kAggDense, kCap, kSearch>(vec), reduce_kernel<kAggSgd, kCap, kSearch>(vec),
+          reduce_kernel<kAggMomentum, kCap, kSearch>(vec)})
+      cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout,
+                           cudaSharedmemCarveoutMaxShared);
 }
 }  // namespace
 
@@ -719,8 +737,10 @@ void aggregate_init_device(DeviceInfo& info) {
     per_sm = f == streams[0] || b < per_sm ? b : per_sm;
   }
   info.agg_stream_slots = per_sm * info.sm_count;
-  prefer_shared<kFewWorkers>();
-  prefer_shared<kMaxWorkers>();
+  prefer_shared<kFewWorkers, false>();
+  prefer_shared<kFewWorkers, true>();
+  prefer_shared<kMaxWorkers, false>();
+  prefer_shared<kMaxWorkers, true>();
   cudaGetLastError();
 }
 
