@@ -27,6 +27,7 @@
 #include <algorithm>
 #include <cstddef>
 
+#include "agg_rule.h"
 #include "internal.h"
 #include "tma.cuh"
 
@@ -46,7 +47,7 @@ struct AggPtrs {
 
 // off[i * (tiles + 1) + t] = number of entries of list i below t * kAggTile;
 // off[i * (tiles + 1) + tiles] = counts[i]. Grid: blockIdx.y = list, x over
-// the tiles + 1 entries. Two ways to the same numbers:
+// the tiles + 1 entries. Two ways to the same numbers (agg_rule.h):
 //  - scattered, when the lists hold at most kScatterEntries entries together
 //    and this one at least (tiles + 1) / 16: entry p (p = 0..count, count
 //    standing for the end) owns the tiles t with
@@ -59,12 +60,6 @@ struct AggPtrs {
 // ascending is latched as bad input (scatter) and may leave entries the
 // reduction clamps to the list. A strictly ascending list below d has at most
 // d entries: a larger count is latched, and nothing past d entries is read.
-// The scatter reads every index once (32 MB at most, about 8 us), the searches
-// take 8 to 12 us whatever the lists hold. Measured, us an exchange, searches
-// -> scatter: 16 lists of 256 K entries over 6,240 tiles 61.6 -> 54.8, 4
-// LSTM-shaped workers' steps with their exchange (0.9 M entries each) 333.5 ->
-// 300.2.
-constexpr uint32_t kScatterEntries = 8u << 20;
 template <uint32_t kCap>
 __global__ void __launch_bounds__(kThreads)
     agg_offsets_kernel(AggPtrs<kCap> p, const uint32_t* __restrict__ counts, uint32_t n,
@@ -77,14 +72,14 @@ __global__ void __launch_bounds__(kThreads)
   const uint32_t tx = blockIdx.x * kThreads + threadIdx.x;
   const uint32_t stride = gridDim.x * kThreads;  // >= per
   const int lane = threadIdx.x & 31;
-  uint32_t all = 0;  // entries of all lists (each clamped: 256 of them fit)
-  for (uint32_t q = lane; q < n; q += 32) all += min(counts[q], 1u << 23);
+  uint32_t all = 0;  // entries of all lists
+  for (uint32_t q = lane; q < n; q += 32) all += scatter_share(counts[q]);
   all = warp_sum(all);
   const uint32_t cnt = min(counts[i], d);
   if (counts[i] > d && tx == 0) atomicOr(error, kDevErrBadInput);
   const uint32_t* x = p.idx[i];
   uint32_t* o = off + static_cast<uint64_t>(i) * per;
-  if (cnt < per / 16 || all > kScatterEntries) {
+  if (!scatter_offsets(cnt, all, per)) {
     if (tx >= per) return;
     uint32_t result = cnt;
     if (tx < tiles) {

@@ -87,6 +87,28 @@ def test_more_entries_than_the_scatter_takes():
     assert efs.ef_check_status() == efs.EF_OK
 
 
+def test_one_list_of_more_entries_than_the_scatter_takes():
+    # a step that sends 9.4 M pairs from a shifted error memory: its tile index
+    # comes from the list, and so do the offsets of its exchange
+    d = 9_400_003
+    rng = np.random.default_rng(3)
+    g, e = (rng.standard_normal(d).astype(np.float32) for _ in range(2))
+    gd, ed = gu.to_dev(g), gu.to_dev(e, 1)
+    idx = torch.empty(d, dtype=torch.int32, device=gu.DEV)
+    val, dense = torch.empty(d, device=gu.DEV), torch.empty(d, device=gu.DEV)
+    cnt = torch.empty(1, dtype=torch.int32, device=gu.DEV)
+    tt = torch.full((efs.tiles_for(d),), -1, dtype=torch.int32, device=gu.DEV)
+    efs.ef_hard_threshold(gd, ed, 0.1, 1e-6, idx, val, cnt, tiles_out=tt)
+    ri, rv, _ = oracle.ef_hard_threshold(g, e, 0.1, 1e-6)
+    assert int(cnt.item()) == ri.size > 8 << 20
+    edges = np.arange(efs.tiles_for(d) - 1, dtype=np.int64) * TILE
+    gu.assert_bits(tt.cpu().numpy(), np.append(np.searchsorted(ri.astype(np.int64), edges),
+                                               ri.size).astype(np.int32), "tiles")
+    efs.sparse_aggregate([idx], [val], cnt, d, dense)
+    gu.assert_bits(dense.cpu().numpy(), oracle.sparse_aggregate([ri], [rv], d), "sum")
+    assert efs.ef_check_status() == efs.EF_OK
+
+
 def test_malformed_lists_many_tiles():
     # a tile index that sends a tile another tile's pairs, and an index past d:
     # skipped and latched, every other coordinate as if they were absent
