@@ -12,11 +12,17 @@
 
 namespace efs {
 
-// The scatter reads every index once (32 MB at most, about 8 us), the searches
-// take 8 to 12 us whatever the lists hold. Measured, us an exchange, searches
-// -> scatter: 16 lists of 256 K entries over 6,240 tiles 61.6 -> 54.8, 4
-// LSTM-shaped workers' steps with their exchange (0.9 M entries each) 333.5 ->
-// 300.2; one list of 34.6 M entries over 33,779 tiles 159 -> 180.
+// The scatter's time grows with the entries it reads, the searches' with the
+// number of lists and tiles. Measured on a GB300, us an exchange, searches ->
+// scatter, by entries a tile and list:
+//     41  16 lists over 6,240 tiles 60.2 -> 48.7, over 33,779 217 -> 203,
+//         256 lists over 1,954 527 -> 518, 4 over 33,779 122.4 -> 118.3
+//      4  64 lists over 33,779 tiles 652 -> 629
+//    164  4 lists over 33,779 tiles 148.3 -> 153.5, 1 over 6,240 30.4 -> 23.2
+//   1024  1 list over 33,779 tiles 159 -> 180, 4 over 1,954 34.9 -> 36.6
+// So a list of up to 64 entries a tile is scattered, and every list while they
+// are few together (32 MB of indexes, about 8 us).
+constexpr uint32_t kScatterPerTile = 64;
 constexpr uint32_t kScatterEntries = 8u << 20;
 
 // A list's entries as they are summed over all lists: 256 of them fit 32 bits,
@@ -28,7 +34,8 @@ EFS_HOST_DEVICE uint32_t scatter_share(uint32_t count) {
 // Scatter a list of `count` entries over `per` offsets? `all` is the sum of
 // the lists' shares.
 EFS_HOST_DEVICE bool scatter_offsets(uint32_t count, uint32_t all, uint32_t per) {
-  return count >= per / 16 && all <= kScatterEntries;
+  const bool few = count / kScatterPerTile < per || all <= kScatterEntries;
+  return count >= per / 16 && few;
 }
 
 }  // namespace efs

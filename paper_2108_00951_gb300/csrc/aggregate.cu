@@ -48,12 +48,13 @@ struct AggPtrs {
 // off[i * (tiles + 1) + t] = number of entries of list i below t * kAggTile;
 // off[i * (tiles + 1) + tiles] = counts[i]. Grid: blockIdx.y = list, x over
 // the tiles + 1 entries. Two ways to the same numbers (agg_rule.h):
-//  - scattered, when the lists hold at most kScatterEntries entries together
-//    and this one at least (tiles + 1) / 16: entry p (p = 0..count, count
-//    standing for the end) owns the tiles t with
-//    list[p - 1] < t * kAggTile <= list[p] and writes p there. A thread reads
-//    4 consecutive entries and the one before them, nothing waits for
-//    anything else; a run of more than 8 tiles is written by the whole warp;
+//  - scattered, when this list holds up to kScatterPerTile entries a tile, or
+//    the lists at most kScatterEntries together, and this one at least
+//    (tiles + 1) / 16: entry p (p = 0..count, count standing for the end) owns
+//    the tiles t with list[p - 1] < t * kAggTile <= list[p] and writes p
+//    there. A thread reads 4 consecutive entries and the one before them,
+//    nothing waits for anything else; a run of more than 8 tiles is written by
+//    the whole warp;
 //  - otherwise one binary search per tile (14-23 dependent loads, but
 //    independent of the lists' length).
 // Either way every entry lies in [0, count]; a list that is not strictly

@@ -44,7 +44,15 @@ def test_one_list_can_hold_too_many(scattered):
 
 def test_many_long_lists_do_not_wrap_the_sum(scattered):
     assert not any(scattered([2**32 - 1] * 256, 33_779))
-    assert not any(scattered([16 << 20] * 255 + [300_000], 33_779))
+    assert not any(scattered([16 << 20] * 255 + [300_000], 4_000))
+
+
+def test_many_lists_of_few_entries_a_tile_are_scattered(scattered):
+    # 9 M entries together, but 2.2 M searches: 64 lists of 0.1 % of 138.4 M
+    assert all(scattered([140_000] * 64, 33_779))
+    assert all(scattered([8 * 33_780] * 256, 33_779))
+    # each list by its own length
+    assert scattered([64 * 33_780 - 1, 64 * 33_780] + [7 << 20], 33_779) == [True, False, False]
 
 
 def test_sparse_lists_are_searched(scattered):

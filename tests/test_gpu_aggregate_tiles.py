@@ -87,6 +87,19 @@ def test_more_entries_than_the_scatter_takes():
     assert efs.ef_check_status() == efs.EF_OK
 
 
+def test_many_lists_some_scattered_and_some_searched():
+    # over 8 M entries together: lists of up to 64 a tile are scattered, the
+    # longest and the shortest searched
+    d = 1300 * TILE - 5
+    two, twov = _lists(d, [75_000, 60_000], 5)
+    other, otherv = _lists(d, [300_000, 30], 6)
+    other[1], otherv[1] = other[1][:70], otherv[1][:70]
+    idx, val = two * 60 + other, twov * 60 + otherv
+    assert sum(i.size for i in idx) > 8 << 20
+    gu.assert_bits(_sum(idx, val, d, False), oracle.sparse_aggregate(idx, val, d), "mixed lists")
+    assert efs.ef_check_status() == efs.EF_OK
+
+
 def test_one_list_of_more_entries_than_the_scatter_takes():
     # a step that sends 9.4 M pairs from a shifted error memory: its tile index
     # comes from the list, and so do the offsets of its exchange
