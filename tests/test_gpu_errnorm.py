@@ -3,8 +3,8 @@ against the oracle's fp64 sum of the oracle's own residual.
 
 Tolerance, derived from the arithmetic (every partial sum of nonnegative fp32
 squares sees at most 13 roundings, then fp64): relative 1e-6. Every route of
-every step is reached: the hard-threshold stream and its look-back fallback
-for misaligned inputs; entire-vector Top-k with a short candidate list, a list
+every step is reached: the hard-threshold stream, aligned and over the shifted
+tiles of misaligned inputs; entire-vector Top-k with a short candidate list, a list
 beyond shared memory, the full-array mode, k = 0 and k = d, misaligned
 inputs; layer-wise Top-k over every kind of segment, teams, selection from e,
 a cut-off list and misaligned inputs. Requesting the norm leaves every other

@@ -118,7 +118,7 @@ def test_ht_zero_length():
 @pytest.mark.parametrize("off", [0, 1])
 def test_ht_concurrent_streams(off):
     # calls on different streams use different workspaces and may overlap
-    # (off = 1: misaligned bases, the look-back kernel and its tile dispenser)
+    # (off = 1: misaligned bases, the same kernels over shifted tiles)
     d = 300_000
     g1, e1 = _inputs(d, 4)
     g2, e2 = _inputs(d, 5)
@@ -178,10 +178,11 @@ def test_topk_concurrent_streams(kind):
     assert efs.ef_check_status() == efs.EF_OK
 
 
-def test_ht_lookback_dispenser_back_to_back():
-    # the look-back kernel (misaligned bases) takes its tile ids from a
-    # per-stream dispenser that the last CTA to finish leaves at zero: launches
-    # of different tile counts in a row on one stream, each equal to the oracle
+@pytest.mark.usefixtures("ht_stream_kernel")
+def test_ht_shifted_back_to_back():
+    # misaligned bases stream through shifted tiles; launches of different tile
+    # counts in a row on one stream, each equal to the oracle (the one-tile-
+    # per-CTA kernel's dispenser: test_noalloc_dispenser_back_to_back)
     for r, d in enumerate([5 * 4096 + 3, 1, 4096, 700_001, 3 * 4096 + 17, 2 * 4096]):
         g, e = _inputs(d, 30 + r)
         _check_same(gu.ht(g, e, 0.1, 1.5e-3, g_off=1, e_off=1),

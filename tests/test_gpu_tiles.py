@@ -1,6 +1,6 @@
 """The tile index of a message (uint32[ceil(d / 4096) + 1]: the pairs below
 each multiple of 4096, then the count): written by ef_hard_threshold_tiled
-(streaming path, and the look-back path for misaligned inputs), consumed by
+(by the streaming kernel, or for a shifted e from the finished list), consumed by
 the tiled aggregation entries, which must give the same results as the
 searching ones. The expected tile index is the definition evaluated on the
 oracle's index list (np.searchsorted); the sums are the oracle's."""
@@ -78,7 +78,7 @@ def test_hard_threshold_writes_the_tile_index(d, bf16):
 @pytest.mark.parametrize("offs", [(0, 0), (1, 0)])
 def test_tile_index_with_the_error_norm(offs):
     # both optional outputs of ef_hard_threshold_tiled at once, on the
-    # streaming and on the misaligned path; the norm within the relative
+    # aligned and on the misaligned path; the norm within the relative
     # 1e-6 of the error-norm tests, the other outputs bit-exact
     d = 3 * 2**20 + 4099
     g, e = _inputs(d, 3)

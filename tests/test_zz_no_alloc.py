@@ -122,6 +122,39 @@ def test_noalloc_allocates_no_device_memory():
     assert int(status.item()) == 0
 
 
+def test_noalloc_dispenser_back_to_back():
+    # the one-tile-per-CTA kernel takes its tiles from a dispenser in the fixed
+    # scratch that the last CTA to finish leaves at zero: launches of different
+    # tile counts in a row, none waited for, each equal to the oracle
+    fn = _entry()
+    dev = torch.device("cuda:0")
+    stream = torch.cuda.current_stream()
+    calls = []
+    for r, d in enumerate([5 * 4096 + 3, 1, 4096, 700_001, 3 * 4096 + 17, 2 * 4096]):
+        rng = np.random.default_rng(30 + r)
+        g = (rng.standard_normal(d) * 1e-2).astype(np.float32)
+        e = (rng.standard_normal(d) * 1e-3).astype(np.float32)
+        off = r % 2
+        calls.append((g, e, gu.to_dev(g, off), gu.to_dev(e, off),
+                      torch.full((d,), -1, dtype=torch.int32, device=dev),
+                      torch.zeros(d, device=dev),
+                      torch.full((1,), -1, dtype=torch.int32, device=dev),
+                      torch.full((1,), 9, dtype=torch.int32, device=dev)))
+    torch.cuda.synchronize()
+    for _, _, gd, ed, idx, val, cnt, status in calls:
+        assert _noalloc(fn, gd, ed, 0.1, 1.5e-3, idx, val, cnt, status, stream) == efs.EF_OK
+    torch.cuda.synchronize()
+    for g, e, gd, ed, idx, val, cnt, status in calls:
+        ri, rv, re_ = oracle.ef_hard_threshold(g, e, 0.1, 1.5e-3)
+        what = "back to back d=%d" % g.size
+        assert int(status.item()) == 0, what
+        c = int(cnt.item())
+        assert c == ri.size, what
+        gu.assert_bits(_bits(idx[:c]), ri, what + " idx")
+        gu.assert_bits(val[:c].cpu().numpy(), rv, what + " val")
+        gu.assert_bits(ed.cpu().numpy(), re_, what + " e'")
+
+
 def test_noalloc_status_reports_a_wait_that_ran_out():
     fn = _entry()
     dev = torch.device("cuda:0")
