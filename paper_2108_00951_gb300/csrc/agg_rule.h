@@ -15,11 +15,12 @@ namespace efs {
 // The scatter's time grows with the entries it reads, the searches' with the
 // number of lists and tiles. Measured on a GB300, us an exchange, searches ->
 // scatter, by entries a tile and list:
-//     41  16 lists over 6,240 tiles 60.2 -> 48.7, over 33,779 217 -> 203,
-//         256 lists over 1,954 527 -> 518, 4 over 33,779 122.4 -> 118.3
-//      4  64 lists over 33,779 tiles 652 -> 629
-//    164  4 lists over 33,779 tiles 148.3 -> 153.5, 1 over 6,240 30.4 -> 23.2
-//   1024  1 list over 33,779 tiles 159 -> 180, 4 over 1,954 34.9 -> 36.6
+//     41  16 lists over 6,240 tiles 49.3 -> 49.1, over 33,779 218 -> 202,
+//         256 lists over 1,954 520 -> 510, 4 over 33,779 122.3 -> 119.2
+//      4  64 lists over 33,779 tiles 655 -> 627
+//    164  4 lists over 33,779 tiles 147.9 -> 154.8, 16 over 6,240 77.0 -> 83.7,
+//         1 over 6,240 29.3 -> 23.6
+//   1024  1 list over 33,779 tiles 153 -> 180, 16 over 1,954 80 -> 114
 // So a list of up to 64 entries a tile is scattered, and every list while they
 // are few together (32 MB of indexes, about 8 us).
 constexpr uint32_t kScatterPerTile = 64;
