@@ -65,14 +65,15 @@
  * DIFFERENT streams never share a workspace and may run concurrently; calls
  * on the same stream are ordered by the stream.
  *
- * Concurrency: below 4096 tiles (16,777,216 coordinates) the streaming
- * kernel's CTAs wait (bounded) only for lower-numbered CTAs of the same
- * launch, which the device dispatches first; kernels that wait on every CTA
+ * Concurrency: below 4096 tiles (16,777,216 coordinates; a dense hard-threshold
+ * call below 1024, see ef_test_set_stream_kernel) the streaming kernel's CTAs
+ * wait (bounded) only for lower-numbered CTAs of the same launch, which the
+ * device dispatches first; kernels that wait on every CTA
  * of their grid (the Top-k select, the layer-wise select with teams) are
  * cooperative launches. If kernels on other streams or other processes (MPS)
  * hold SMs long enough that a CTA cannot start within the bound (2 s), the
  * call fails with EF_ERR_TIMEOUT (reported by ef_check_status); it never
- * hangs and never returns a wrong result. From 4096 tiles on, the streaming
+ * hangs and never returns a wrong result. From there on, the streaming
  * kernel's CTAs claim groups of tiles in the order they start, and the
  * one-tile-per-CTA kernel (ef_hard_threshold_noalloc) takes its tiles the same
  * way: neither needs co-residency.
@@ -348,10 +349,12 @@ ef_status sparse_aggregate_apply(uint32_t n, const uint32_t* const* idx,
  * index is uint32[T + 1] with
  *     tiles[t] = the number of its pairs with index < EF_TILE * t, t < T,
  *     tiles[T] = its count.
- * The aggregation works tile by tile and otherwise finds these positions by a
- * binary search of every list at every tile boundary (one more kernel, whose
- * chains of dependent loads make it latency-bound); the hard-threshold kernel
- * knows them as it places the pairs and writes them for T + 1 words. A worker
+ * The aggregation works tile by tile and otherwise finds these positions
+ * itself: up to 911 tiles by a search at the start of each tile, beyond with one
+ * more kernel that reads every index (lists of few entries a tile) or searches
+ * each list at every tile boundary (the others). The hard-threshold kernel
+ * knows them as it places the pairs and writes them for T + 1 words (with an e
+ * that is not 16-byte aligned, one more kernel finds them in the list). A worker
  * can send the tile index with its message (4 (T + 1) bytes against 8 bytes per
  * pair).
  *

@@ -22,7 +22,7 @@ constexpr size_t kOffGroupErr = 32;     // uint32[2]: with an error norm: groups
                                         // finished (zero between calls)
 constexpr size_t kOffGroupCaptured = 40;  // uint32: groups handed out, of captured calls
 constexpr size_t kOffTkListCount = 72;  // uint32: candidates emitted by the streaming pass
-constexpr size_t kOffErrArrive = 80;    // uint32: arrivals of the e' norm pass (zero after it)
+constexpr size_t kOffErrArrive = 80;    // uint32: CTAs of a rounding step that finished (zero after it)
 constexpr size_t kOffRoundTotal = 84;   // uint32: coordinates the rounding did not send (zero after it)
 constexpr size_t kOffStreamErr = 88;    // double: the streaming pass's share of ||e'||^2
 // Per-call Top-k state that must start at zero, in two blocks used by

@@ -281,8 +281,8 @@ __global__ void __launch_bounds__(kLbThreads, 1)
   if (threadIdx.x < kSWarps) s_freed[threadIdx.x] = 0;
   __syncthreads();
   // A dependent launch starts while the previous kernel's last groups are
-  // placed, a phase that leaves DRAM mostly idle: pull the first groups the
-  // CTAs will claim (about two each, claimed in CTA order) toward L2
+  // placed, a phase that leaves DRAM mostly idle: pull the first groups that
+  // will be claimed (two for every CTA, whichever takes them) toward L2
   // meanwhile. A prefetch is not a read of the data: L2 is the point of
   // coherence, so the previous kernel's writes still land before the bulk
   // copies read these lines. Whole tiles only.
