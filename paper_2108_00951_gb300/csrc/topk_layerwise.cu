@@ -621,9 +621,23 @@ __device__ bool select_team(const LwArgs& a, const LwSeg& s, const SegHead& head
                             bool& overflow, bool& bad, uint32_t* s_hist, uint32_t* s_w,
                             ErrAcc* err) {
   __shared__ uint32_t s_found, s_last;
+  __shared__ Source s_src;
+  __shared__ uint32_t s_from;
   const int tid = threadIdx.x;
-  const Source src = segment_source(a, s, head);
-  const uint32_t err_from = err_from_for(s, head.bound, src.list);
+  // The same for every thread, but taken from shared memory: left in the
+  // registers that the head's loads filled, it made the loops over a long
+  // source slower. us a call, VGG-16-shaped: at 3 % 6,210 -> 5,775, at 5 % 6,470
+  // -> 6,100 (before the head was read in one round trip 5,940 and 6,225).
+  {
+    const Source x = segment_source(a, s, head);
+    if (tid == 0) {
+      s_src = x;
+      s_from = err_from_for(s, head.bound, x.list);
+    }
+  }
+  __syncthreads();
+  const Source src = s_src;
+  const uint32_t err_from = s_from;
   const float* vals = src.list ? a.list_val + src.c0 : e + s.lo;
   const uint32_t* idxs = src.list ? a.list_idx + src.c0 : nullptr;
   const MagsGlobal mag{vals};
