@@ -8,8 +8,8 @@
 // and no singles' CTA (but for one long single). The load starts at
 // kLwRankLoad and grows until teams and singles fit the CTAs there are.
 // Teams that took all but one CTA left the singles to it one after another:
-// us a call, ResNet-50-shaped at 5 %, 143 singles, 1,285 -> 348; VGG-16-shaped
-// at 5 % 12,500 -> 6,500; 138 M coordinates in 200 tensors at 1 % 2,304 -> 383.
+// us a call, ResNet-50-shaped at 5 %, 143 singles, 1,285 -> 339; VGG-16-shaped
+// at 5 % 12,500 -> 6,080; 138 M coordinates in 200 tensors at 1 % 2,304 -> 383.
 #pragma once
 
 #include <algorithm>
